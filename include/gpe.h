@@ -289,8 +289,9 @@ gpe_status gpe_density_adjoint(gpe_ctx* ctx, const void* phi_dev, const double* 
 
 /* Thomas-Fermi initial data (Section 6, eq. TF_App): phi_0 = sqrt(max(mu - V, 0) / eta),
  * with mu fixed by the normalisation h^d sum max(mu - V, 0) / eta = 1 (so that
- * ||phi_0|| = 1), found by bisection on the device (120 halvings of the bracket
- * [min V, max V + eta / (h^d N)]).  The closed forms of eq. TF_Rdius hold for
+ * ||phi_0|| = 1), found on the device by Newton's method on this convex,
+ * piecewise linear function of mu, bounded by bisection of the bracket
+ * [min V, max V + eta / (h^d N)] (at most 240 sweeps over V).  The closed forms of eq. TF_Rdius hold for
  * the paper's harmonic traps only; the normalisation holds for any V.
  *  phi_out : complex128 [z][y][x], host or device.
  *  mu_out  : may be NULL; receives mu.

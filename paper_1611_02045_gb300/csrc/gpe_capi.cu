@@ -77,7 +77,7 @@ struct gpe_ctx {
                          // 16 (streaming form) by default in single precision for n >= 64
   double vmax = 0.0;  // max V on the grid
   double vmin = 0.0;  // min V on the grid
-  double* tf_state = nullptr;  // Thomas-Fermi bisection bracket (2 doubles, device)
+  TfState* tf_state = nullptr;  // Thomas-Fermi root search (device)
   int max_threads[2] = {512, 256};
   bool warmed[3] = {false, false, false};  // per launch mode
   int nsm = 0;                      // streaming multiprocessors of the device
@@ -517,21 +517,31 @@ extern "C" gpe_status gpe_thomas_fermi(gpe_ctx* c, void* phi_out, double* mu_out
   if (!c) return GPE_ERR_ARG;
   if (!phi_out) { c->err = "null phi"; return GPE_ERR_ARG; }
   if (!(c->prob.eta > 0.0)) { c->err = "the Thomas-Fermi state needs eta > 0"; return GPE_ERR_ARG; }
-  if (!c->tf_state) GPE_CU(c, cudaMalloc(&c->tf_state, 2 * sizeof(double)));
-  // bracket: S(vmin) = 0 < 1 and S(vmax + eta / (h^d N)) >= 1
-  const double br[2] = {c->vmin, c->vmax + c->prob.eta / (c->weight * (double)c->N)};
-  GPE_CU(c, cudaMemcpyAsync(c->tf_state, br, sizeof(br), cudaMemcpyHostToDevice, c->st));
+  if (!c->tf_state) GPE_CU(c, cudaMalloc(&c->tf_state, sizeof(TfState)));
+  // bracket: S(vmin) = 0 < 1 and S(vmax + eta / (h^d N)) >= 1; Newton starts from its right end
+  TfState S;
+  S.lo = c->vmin;
+  S.hi = S.x = c->vmax + c->prob.eta / (c->weight * (double)c->N);
+  S.dx = 1.7976931348623157e308;
+  S.done = 0;
+  const TfState init = S;
   const double* V64 = static_cast<const double*>(c->pb[1].V);
-  for (int it = 0; it < 120; ++it)  // halves the bracket each time: far below one ulp of mu
-    GPE_CU(c, launch_tf_bisect(V64, c->N, c->weight, c->prob.eta, c->tf_state, c->partials, c->ticket, c->st));
+  // Newton needs about 8 sweeps for the usual traps and at least every second one halves
+  // the bracket otherwise; the host looks every kTfCheck sweeps
+  constexpr int kTfCheck = 10, kTfMost = 240;
+  for (int it = 0; it < kTfMost && !S.done; it += kTfCheck) {
+    for (int k = 0; k < kTfCheck; ++k)
+      GPE_CU(c, launch_tf_step(V64, c->N, c->weight / c->prob.eta, c->tf_state, init, it + k == 0, c->partials,
+                               c->ticket, c->st));
+    GPE_CU(c, cudaMemcpyAsync(&S, c->tf_state, sizeof(S), cudaMemcpyDeviceToHost, c->st));
+    GPE_CU(c, cudaStreamSynchronize(c->st));
+  }
   const bool dev = is_device_ptr(phi_out);
   void* dst = dev ? phi_out : c->pb[1].phi;
   GPE_CU(c, launch_tf_fill(V64, c->N, c->prob.eta, c->tf_state, dst, c->st));
   if (!dev) GPE_CU(c, cudaMemcpyAsync(phi_out, dst, 16 * (size_t)c->N, cudaMemcpyDeviceToHost, c->st));
-  double st[2];
-  GPE_CU(c, cudaMemcpyAsync(st, c->tf_state, sizeof(st), cudaMemcpyDeviceToHost, c->st));
   GPE_CU(c, cudaStreamSynchronize(c->st));
-  if (mu_out) *mu_out = 0.5 * (st[0] + st[1]);
+  if (mu_out) *mu_out = S.x;
   return GPE_OK;
 }
 

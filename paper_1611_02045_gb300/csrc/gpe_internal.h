@@ -245,11 +245,19 @@ cudaError_t launch_batch_gate64(Ctl* ctl, unsigned long long cond, cudaStream_t 
 cudaError_t prepare_cluster_solve(int M);
 
 // Thomas-Fermi initial data (eq. TF_App): mu solving h^d sum max(mu - V, 0) / eta = 1
-// by bisection (state[0] = lo, state[1] = hi on entry; each launch halves the
-// bracket), then phi = sqrt(max(mu - V, 0) / eta) as complex128.
-cudaError_t launch_tf_bisect(const double* V, long long n, double weight, double eta, double* state,
-                             double* partials, unsigned* ticket, cudaStream_t st);
-cudaError_t launch_tf_fill(const double* V, long long n, double eta, const double* state, void* phi128,
+// inside the bracket [lo, hi] by Newton's method with bisection as its bound
+// (each launch is one step; done: later launches change nothing), then
+// phi = sqrt(max(mu - V, 0) / eta) as complex128 with mu = state->x.
+// The first launch starts from init, the others from *state.  w_eta: h^d / eta.
+// partials: >= 2048 doubles of scratch.
+struct TfState {
+  double lo, hi, x;
+  double dx;  // last Newton step
+  int done;
+};
+cudaError_t launch_tf_step(const double* V, long long n, double w_eta, TfState* state, const TfState& init, bool first,
+                           double* partials, unsigned* ticket, cudaStream_t st);
+cudaError_t launch_tf_fill(const double* V, long long n, double eta, const TfState* state, void* phi128,
                            cudaStream_t st);
 
 // Spectral interpolation onto a grid twice as fine along one axis

@@ -25,14 +25,18 @@ namespace gpe {
 
 namespace {
 
-template <int Mc>
+// STR: lines a field row apart (y, z).  Neighbouring threads then hold neighbouring
+// lines (tid = l + lpb t), so that lpb adjacent columns fill whole memory sectors;
+// along x they hold neighbouring points of one line (tid = t + Tl l).
+template <int Mc, bool STR>
 __global__ void __launch_bounds__(256) k_interp(InterpArgs a) {
   constexpr int Mf = 2 * Mc, Tl = Mc / 4;
   constexpr int LS = Mf + Mf / 16;
   extern __shared__ __align__(16) unsigned char smraw[];
   double2* sm = reinterpret_cast<double2*>(smraw);
-  const int t = threadIdx.x % Tl, l = threadIdx.x / Tl;
-  const long long line = (long long)blockIdx.x * (blockDim.x / Tl) + l;  // grid covers the lines exactly
+  const int lpb = blockDim.x / Tl;
+  const int t = STR ? threadIdx.x / lpb : threadIdx.x % Tl, l = STR ? threadIdx.x % lpb : threadIdx.x / Tl;
+  const long long line = (long long)blockIdx.x * lpb + l;  // grid covers the lines exactly
   const long long inner = line % a.inner_count, outer = line / a.inner_count;
   const double2* __restrict__ in = a.in + outer * a.in_outer + inner * a.in_inner;
   double2* __restrict__ out = a.out + outer * a.out_outer + inner * a.out_inner;
@@ -59,36 +63,49 @@ __global__ void __launch_bounds__(256) k_interp(InterpArgs a) {
   for (int q = 0; q < 8; ++q) out[(long long)(t + q * Tl) * a.out_stride] = vf[q];
 }
 
-template <int Mc>
+// Lines per block: an FP64 warp instruction holds its SM sub-partition's FP64
+// pipe for 64 cycles, so the pass takes as long as the busiest of the 608
+// sub-partitions: the fewest lines per block that still make a warp (and, for
+// strided lines, a 32-byte sector of two columns) spread the warps best.
+// 256^2 -> 512^2, x axis: 25.3 us in 64 blocks of 256 threads, 13.4 us in 256
+// blocks (its FP64 instructions alone take about 10 us); y axis 25 us in either
+// (twice the lines: the FP64 pipes are busy for about 21 us).
+template <int Mc, bool STR>
 cudaError_t launch_interp_one(const InterpArgs& a, cudaStream_t st) {
   constexpr int Tl = Mc / 4, LS = 2 * Mc + 2 * Mc / 16;
   long long lpb = 256 / Tl;
   if (lpb < 1) lpb = 1;
-  while (lpb > 1 && a.lines % lpb != 0) lpb >>= 1;
+  const long long least = Tl >= 32 ? (STR ? 2 : 1) : 32 / Tl;
+  while (lpb > 1 && (a.lines % lpb != 0 || (lpb > least && a.lines / lpb < 8 * 152))) lpb >>= 1;
   const size_t smem = (size_t)lpb * LS * sizeof(double2);
   static DeviceOnce attr;
   const int dev = DeviceOnce::device();
   if (!attr.done(dev)) {
-    const cudaError_t e = cudaFuncSetAttribute(k_interp<Mc>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+    const cudaError_t e = cudaFuncSetAttribute(k_interp<Mc, STR>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
     if (e != cudaSuccess) return e;
     attr.set(dev);
   }
-  k_interp<Mc><<<(unsigned)(a.lines / lpb), (unsigned)(Tl * lpb), smem, st>>>(a);
+  k_interp<Mc, STR><<<(unsigned)(a.lines / lpb), (unsigned)(Tl * lpb), smem, st>>>(a);
   return cudaGetLastError();
 }
 
 }  // namespace
 
-cudaError_t launch_interp(int Mc, const InterpArgs& a, cudaStream_t st) {
+template <bool STR>
+static cudaError_t launch_interp_axis(int Mc, const InterpArgs& a, cudaStream_t st) {
   switch (Mc) {
-    case 8: return launch_interp_one<8>(a, st);
-    case 16: return launch_interp_one<16>(a, st);
-    case 32: return launch_interp_one<32>(a, st);
-    case 64: return launch_interp_one<64>(a, st);
-    case 128: return launch_interp_one<128>(a, st);
-    case 256: return launch_interp_one<256>(a, st);
+    case 8: return launch_interp_one<8, STR>(a, st);
+    case 16: return launch_interp_one<16, STR>(a, st);
+    case 32: return launch_interp_one<32, STR>(a, st);
+    case 64: return launch_interp_one<64, STR>(a, st);
+    case 128: return launch_interp_one<128, STR>(a, st);
+    case 256: return launch_interp_one<256, STR>(a, st);
     default: return cudaErrorInvalidValue;
   }
+}
+
+cudaError_t launch_interp(int Mc, const InterpArgs& a, cudaStream_t st) {
+  return a.in_stride == 1 ? launch_interp_axis<false>(Mc, a, st) : launch_interp_axis<true>(Mc, a, st);
 }
 
 }  // namespace gpe
