@@ -64,7 +64,7 @@ struct gpe_ctx {
   Ctl* ctl_solve = nullptr;
   Ctl* ctl_api = nullptr;
   double* partials = nullptr;
-  unsigned* ticket = nullptr;
+  unsigned* ticket = nullptr;  // [0] reduction ticket, [1..3] blocks in each region of the partials
   double* log_dev = nullptr;
   int log_dev_cap = 0;
   PassPlan plan[3];      // default plan per axis (E = 8, heuristic widths)
@@ -149,10 +149,13 @@ static PassArgs base_args(gpe_ctx* c, int prec, int axis, int mode) {
   a.axis = axis; a.M = pl.M; a.E = pl.E; a.lpb = pl.lpb; a.tx = pl.tx; a.stride = pl.stride;
   a.outer_stride = pl.outer_stride; a.ntx = pl.ntx; a.nblocks = pl.nblocks;
   a.weight = c->weight; a.eta = c->prob.eta; a.omega = c->prob.omega;
+  a.eta_n = num(a.eta); a.omega_n = num(a.omega); a.invN = num(1.0 / (double)c->N);
   for (int i = 0; i < 3; ++i) { a.xi[i] = b.xi[i]; a.xc[i] = b.xc[i]; }
   a.tw = b.tw[axis];
   a.V = b.V;
   a.partials = c->partials;
+  a.region = (long long)kMaxMoments * c->partials_cap;
+  a.nparts = reinterpret_cast<int*>(c->ticket) + 1;
   a.ticket = c->ticket;
   return a;
 }
@@ -350,8 +353,8 @@ extern "C" gpe_status gpe_create(const gpe_problem* prob, const double* V, void*
   }
   c->partials_cap = maxblocks > kPlanMaxBlocks ? maxblocks : kPlanMaxBlocks;  // room for tuned plans
   if (cudaMalloc(&c->ctl_solve, sizeof(Ctl)) != cudaSuccess || cudaMalloc(&c->ctl_api, sizeof(Ctl)) != cudaSuccess ||
-      cudaMalloc(&c->partials, sizeof(double) * kMaxMoments * (size_t)c->partials_cap) != cudaSuccess ||
-      cudaMalloc(&c->ticket, sizeof(unsigned)) != cudaSuccess) {
+      cudaMalloc(&c->partials, sizeof(double) * 3 * kMaxMoments * (size_t)c->partials_cap) != cudaSuccess ||
+      cudaMalloc(&c->ticket, 4 * sizeof(unsigned)) != cudaSuccess) {
     c->err = "cudaMalloc workspace"; return fail(GPE_ERR_CUDA);
   }
   {
@@ -366,7 +369,7 @@ extern "C" gpe_status gpe_create(const gpe_problem* prob, const double* V, void*
   }
   cudaMemset(c->ctl_solve, 0, sizeof(Ctl));
   cudaMemset(c->ctl_api, 0, sizeof(Ctl));
-  cudaMemset(c->ticket, 0, sizeof(unsigned));
+  cudaMemset(c->ticket, 0, 4 * sizeof(unsigned));
   if (cudaDeviceSynchronize() != cudaSuccess) { c->err = "set-up failed"; return fail(GPE_ERR_CUDA); }
   *out = c;
   return GPE_OK;
@@ -612,7 +615,7 @@ static gpe_status run_PC(gpe_ctx* c, const IterBufs& b, const void* r, double al
                          bool solver, cudaStream_t st) {
   PassArgs a = base_args(c, b.tab_d, 0, b.mode);
   a.V = b.V;
-  a.ctl = ctl; a.solver = solver; a.phi = b.phi; a.r_in = r; a.api_alpha = alpha;
+  a.ctl = ctl; a.solver = solver; a.phi = b.phi; a.r_in = r; a.api_alpha = num(alpha);
   a.s = b.s; a.t = b.t; a.r_prev = b.r_prev; a.p = b.p; a.out = out;
   GPE_CU(c, launch(b.mode, P_C1, a, st));
   if (c->dim == 3) {
@@ -621,7 +624,7 @@ static gpe_status run_PC(gpe_ctx* c, const IterBufs& b, const void* r, double al
     GPE_CU(c, launch(b.mode, P_CFWD, y, st));
   }
   PassArgs k = base_args(c, b.tab_d, c->dim - 1, b.mode);
-  k.ctl = ctl; k.solver = solver; k.s = b.s; k.api_alpha = alpha;
+  k.ctl = ctl; k.solver = solver; k.s = b.s; k.api_alpha = num(alpha);
   GPE_CU(c, launch(b.mode, P_CCORE, k, st));
   if (c->dim == 3) {
     PassArgs y = base_args(c, b.tab_d, 1, b.mode);

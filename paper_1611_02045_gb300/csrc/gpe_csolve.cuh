@@ -56,7 +56,7 @@ __device__ __forceinline__ void cs_yunit(const cgc::cluster_group& cl, int rank,
   // the last users of xs were the x unit before the reduction's cluster barrier
   line_dft<M, E, -1, false, false>(w, xs, si, t, tw);
   if constexpr (ROLE == P_HMID || ROLE == P_AMID) {
-    const float om = float(a.omega);
+    const float om = a.omega_n.hi;
     const float rx = -static_cast<const float*>(a.xc[0])[x];
     float akin = 0.f, arot = 0.f;  // arot: rotation symbol with omega (A p) or without it (H phi, finalize_H applies it)
 #pragma unroll
@@ -85,7 +85,7 @@ __device__ __forceinline__ void cs_yunit(const cgc::cluster_group& cl, int rank,
     }
   } else {
     static_assert(ROLE == P_CCORE, "y roles: HMID, CCORE, AMID");
-    const float alpha = float(S.alpha);
+    const float alpha = S.alpha.hi;
     const float invN = 1.0f / float(M * M);
     const float kx = static_cast<const float*>(a.xi[0])[x];
     const bool core = pc_core(S.pc);
@@ -104,16 +104,18 @@ __device__ __forceinline__ void cs_yunit(const cgc::cluster_group& cl, int rank,
   }
 }
 
-// Cluster-wide fixed-order sum of the CTAs' block totals (tot[] in FP64,
-// valid in thread 0 of every CTA on return: only thread 0 runs the scalar
+// Cluster-wide fixed-order sum of the CTAs' block totals (tot[] in FP64 and
+// weighted, valid in warp 0 of every CTA on return: only warp 0 runs the scalar
 // steps).  part[2][C][kMaxMoments] lives in CTA 0's shared memory and red_sm
 // holds two block buffers; parity alternates between reductions, so a slow
 // reader never sees the next reduction's partials, and the cluster barrier of
 // the reduction in between orders a buffer's readers before its next writers:
 // no block barrier before the block sum and none after the cluster sum.
-template <int K, unsigned MAXMASK>
+template <int ROLE>
 __device__ __forceinline__ void cs_reduce(const cgc::cluster_group& cl, int rank, int csize, const Acc* acc,
-                                          Acc* part, int& parity, Acc* red_sm, double* tot) {
+                                          Acc* part, int& parity, Acc* red_sm, double weight, double* tot) {
+  constexpr int K = Moments<ROLE>::K;
+  constexpr unsigned MAXMASK = Moments<ROLE>::MAX;
   Acc v[K];
 #pragma unroll
   for (int k = 0; k < K; ++k) v[k] = acc[k];
@@ -130,10 +132,8 @@ __device__ __forceinline__ void cs_reduce(const cgc::cluster_group& cl, int rank
 #pragma unroll
     for (int k = 0; k < K; ++k) v[k] = lane < csize ? p0[lane * kMaxMoments + k] : Acc{0.0f, 0.0f};
     warp_tree<K, MAXMASK>(v);
-    if (lane == 0) {
-#pragma unroll
-      for (int k = 0; k < K; ++k) tot[k] = acc_to_double(v[k]);
-    }
+    totals<K, Moments<ROLE>::W>(v, weight, tot);
+    __syncwarp();
   }
   parity ^= 1;
 }
@@ -154,7 +154,7 @@ __global__ void __launch_bounds__((M / 8) * kCSRows) cluster_solve(ClusterSolveA
   __shared__ Ctl S;
   __shared__ Acc part[2 * kCSRows * kMaxMoments];
   __shared__ Acc red_sm[2 * 32 * kMaxMoments];  // two buffers, alternating with the reductions
-  __shared__ double tot[kMaxMoments];
+  __shared__ double tot[2][kMaxMoments];  // x and y totals of the operator under way
 
   const int row0 = rank * R;
   // load this CTA's rows of phi_0; p_{-1} = r_{-1} = 0
@@ -194,58 +194,42 @@ __global__ void __launch_bounds__((M / 8) * kCSRows) cluster_solve(ClusterSolveA
     for (int k = 0; k < kMaxMoments; ++k) acc[k] = Acc{0.f, 0.f};
   };
 
+  const double w = ax.weight;
   while (!S.done) {
     // ---- H phi_n (x pass folds in the retraction to phi_n) ----
     Scal sc = scal_of(&S, ax);
     zero();
     xunit<float, float, float, M, P_HX>(ax, sc, 0, xsb, acc);
-    cs_reduce<6, 32u>(cl, rank, csize, acc, part, parity, red_sm, tot);
-    if (threadIdx.x == 0)
-      for (int k = 0; k < 6; ++k) S.hsum[0][k] = tot[k];
+    cs_reduce<P_HX>(cl, rank, csize, acc, part, parity, red_sm, w, tot[0]);
     zero();
     cs_yunit<M, P_HMID>(cl, rank, phi_s, t_s, xs, ax, sc, acc);
-    cs_reduce<2, 0u>(cl, rank, csize, acc, part, parity, red_sm, tot);
-    if (threadIdx.x == 0) {
-      S.hsum[1][0] = tot[0];
-      S.hsum[1][1] = tot[1];
-      finalize_H(&S, F, writer);
-    }
+    cs_reduce<P_HMID>(cl, rank, csize, acc, part, parity, red_sm, w, tot[1]);
+    if (threadIdx.x < 32) finalize_H(&S, F, tot[0], tot[1], nullptr, writer);
     __syncthreads();
     // ---- residual, stopping rule, P_C r_n ----
     sc = scal_of(&S, ax);
     zero();
     xunit<float, float, float, M, P_C1>(ax, sc, 0, xsb, acc);
-    cs_reduce<3, 1u>(cl, rank, csize, acc, part, parity, red_sm, tot);
-    if (threadIdx.x == 0) {
-      const double t3[3] = {tot[0], tot[1], tot[2]};
-      finalize_C1(&S, F, t3, writer);
-    }
+    cs_reduce<P_C1>(cl, rank, csize, acc, part, parity, red_sm, w, tot[0]);
+    if (threadIdx.x < 32) finalize_C1(&S, tot[0], writer);
     __syncthreads();
     if (S.done) break;
     cs_yunit<M, P_CCORE>(cl, rank, s_s, nullptr, xs, ax, sc, acc);
     cl.sync();
     zero();
     xunit<float, float, float, M, P_C3>(ax, sc, 0, xsb, acc);
-    cs_reduce<6, 0u>(cl, rank, csize, acc, part, parity, red_sm, tot);
-    if (threadIdx.x == 0) {
-      const double t6[6] = {tot[0], tot[1], tot[2], tot[3], tot[4], tot[5]};
-      finalize_C3(&S, F, t6, writer);
-    }
+    cs_reduce<P_C3>(cl, rank, csize, acc, part, parity, red_sm, w, tot[0]);
+    if (threadIdx.x < 32) finalize_C3(&S, tot[0], writer);
     __syncthreads();
     // ---- p_n and the step size ----
     sc = scal_of(&S, ax);
     zero();
     xunit<float, float, float, M, P_AX>(ax, sc, 0, xsb, acc);
-    cs_reduce<9, 0u>(cl, rank, csize, acc, part, parity, red_sm, tot);
-    if (threadIdx.x == 0)
-      for (int k = 0; k < 9; ++k) S.asum[0][k] = tot[k];
+    cs_reduce<P_AX>(cl, rank, csize, acc, part, parity, red_sm, w, tot[0]);
     zero();
     cs_yunit<M, P_AMID>(cl, rank, p_s, nullptr, xs, ax, sc, acc);
-    cs_reduce<1, 0u>(cl, rank, csize, acc, part, parity, red_sm, tot);
-    if (threadIdx.x == 0) {
-      S.asum[1][1] = tot[0];
-      finalize_A(&S, F, writer);
-    }
+    cs_reduce<P_AMID>(cl, rank, csize, acc, part, parity, red_sm, w, tot[1]);
+    if (threadIdx.x < 32) finalize_A(&S, F, tot[0], tot[1][0], 0.0, writer);
     __syncthreads();
   }
   // write back this CTA's rows of the last iterate and (rank 0) the control block

@@ -24,6 +24,22 @@ struct DeviceOnce {
   }
 };
 
+// A scalar in every kernel precision: d, and its FP32 split hi = (float)d,
+// lo = (float)(d - hi).  On GB300 an FP64 instruction -- a conversion too --
+// holds its SM sub-partition's FP64 pipe for 64 cycles per warp, so kernels
+// read the split made once instead of converting in every warp.
+struct Num {
+  double d;
+  float hi, lo;
+};
+__host__ __device__ inline Num num(double d) {
+  Num n;
+  n.d = d;
+  n.hi = (float)d;
+  n.lo = (float)(d - (double)n.hi);
+  return n;
+}
+
 // Number of doubles in one per-iteration log row (matches GPE_LOG_FIELDS).
 constexpr int kLogFields = 12;
 // Max reduction slots per pass.
@@ -63,17 +79,15 @@ struct Ctl {
   double res_inf, res_l2;
   double rPr, rPr_prev;                 // <r_n, P r_n>, previous
   double beta, gamma;                   // beta_n, Re<d_n, phi_n>
-  double theta, c, s, inv_np, inv_nrm;  // retraction scalars for the next H pass
-  double dE;
+  double theta, dE;
+  // scalars the passes read: the retraction phi <- cc phi + ss p of the next H
+  // pass, lambda_n, the shift lambda~_n, beta_n, gamma_n
+  Num cc, ss, lam_n, alpha_n, beta_n, gamma_n;
   double anchor_res; int anchor_iter;   // stall detection (mixed phase)
   int pad0;
-  double phimax;      // max |phi_n| (H x pass)
+  double umax;        // max |phi_n|^2 (H x pass)
   double floor_coef;  // eps32 (max 1/2|k|^2 + max V): complex64 residual floor per unit |phi|
   double switch_fac;  // complex64 phase ends when ||r||_inf < switch_fac * floor estimate
-  // ---- raw sums written by pass finalisers ----
-  double hsum[3][kMaxMoments];  // H passes, per axis
-  double psum[kMaxMoments];     // P_C passes
-  double asum[3][kMaxMoments];  // A p passes, per axis
   // ---- log ----
   double* log;
   int log_cap;
@@ -112,6 +126,8 @@ struct PassArgs {
   int last_axis;   // 1: this pass is the final one of its operator (runs the finaliser)
   double weight;   // h^d
   double eta, omega;
+  Num eta_n, omega_n;
+  Num invN;        // 1 / number of grid points (a power of two)
   // device tables, in the kernel's precision (T*), stored as void*
   const void* xi[3];   // frequencies per axis, DFT order
   const void* xc[3];   // coordinates per axis
@@ -127,9 +143,11 @@ struct PassArgs {
   void* r_prev;        // r_{n-1}, overwritten with r_n by P_C3 (solver)
   const void* r_in;    // API precond input r
   void* out;           // API output
-  double api_alpha;    // API precond shift (> 0)
+  Num api_alpha;       // API precond shift (> 0)
   Ctl* ctl;
-  double* partials;    // [nblocks][kMaxMoments]
+  double* partials;    // block partials: regions of region doubles (one per axis), [blocks][kMaxMoments] each
+  long long region;
+  int* nparts;         // blocks whose partials each region holds
   unsigned int* ticket;
   unsigned long long cond;  // cudaGraphConditionalHandle (0 = none)
 };
@@ -188,8 +206,8 @@ cudaError_t launch_d2f(const double* src, float* dst, long long n, cudaStream_t 
 cudaError_t launch_d2ds(const double* src, void* dst, long long n, cudaStream_t st);
 cudaError_t launch_convert_c64_to_ds(const void* src, void* dst, long long n, cudaStream_t st);
 cudaError_t launch_convert_ds_to_c128(const void* src, void* dst, long long n, cudaStream_t st);
-// ctl->c = 1, s = 0, inv_nrm = 1 / ||phi||, retract = 1 (weighted norm), so
-// that the next H pass normalises phi in place.
+// ctl->cc = 1 / ||phi||, ss = 0, retract = 1 (weighted norm), so that the next
+// H pass normalises phi in place.
 // prec: 0 complex64, 1 complex128, 2 double-single.
 // partials: >= 1024 doubles of scratch; ticket: the reduction ticket (0 on entry, 0 on exit).
 cudaError_t launch_init_norm(int prec, const void* phi, long long n, double weight, Ctl* ctl, double* partials,

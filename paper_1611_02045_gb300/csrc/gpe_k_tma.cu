@@ -90,7 +90,7 @@ __global__ void __launch_bounds__(512) pass_s_tma(PassArgs a, const __grid_const
   const C* __restrict__ tw = static_cast<const C*>(a.tw);
   const T* __restrict__ xia = tab<T>(a.xi[a.axis]);
   const T invM = T(1) / T(M);
-  const T om = T(a.omega);
+  const T om = num_as<T>(a.omega_n);
   auto si = [tx, c](int pos) { return pos * tx + c; };
 
   if (threadIdx.x == 0 && (long long)blockIdx.x < units) issue(blockIdx.x, 0);
@@ -152,8 +152,8 @@ __global__ void __launch_bounds__(512) pass_s_tma(PassArgs a, const __grid_const
       }
       if constexpr (ROLE == P_CCORE) {
         // (alpha + |k|^2 / 2)^{-1} / N on the full frequency grid (eq. PDelta)
-        const T alpha = T(S.alpha);
-        const T invN = T(1.0 / ((double)a.nx * a.ny * (a.dim == 3 ? a.nz : 1)));
+        const T alpha = num_as<T>(S.alpha);
+        const T invN = num_as<T>(a.invN);
         const T kx = tab<T>(a.xi[0])[ix];
         T kother = 0;
         if (a.dim == 3) {
@@ -241,11 +241,10 @@ __global__ void __launch_bounds__(512) pass_hx_bulk(PassArgs a, int second) {
   const C* __restrict__ tw = static_cast<const C*>(a.tw);
   const T* __restrict__ xi = tab<T>(a.xi[0]);
   const T invM = T(1) / T(M);
-  const T om = T(a.omega), eta = T(a.eta);
+  const T om = num_as<T>(a.omega_n), eta = num_as<T>(a.eta_n);
   auto si = [l](int pos) { return l * LS + pos + (pos >> 4); };
   const bool retract = a.solver && S.retract;
-  const T cc = T(retract ? S.c * S.inv_nrm : 1.0);
-  const T ss = T(retract ? S.s * S.inv_np * S.inv_nrm : 0.0);
+  const T cc = num_as<T>(S.cc), ss = num_as<T>(S.ss);
   C* __restrict__ phi_out = static_cast<C*>(a.phi_out);
   C* __restrict__ tout = static_cast<C*>(a.t);
 

@@ -349,8 +349,7 @@ cudaError_t launch_batch_final(const void* phids, void* phi128, long long n, con
 
 // Fixed-order FP64 sum of |phi|^2 over all blocks (runs once per solve
 // phase): per-block partials, the last block to finish sums them in block
-// order and arms the control block: c = 1, s = 0, inv_nrm = 1 / ||phi||,
-// retract = 1, so that the next H pass normalises phi in place.
+// order and arms the control block: cc = 1 / ||phi||, ss = 0, retract = 1, so that the next H pass normalises phi in place.
 constexpr int kNormThreads = 256;
 template <typename C>
 __global__ void __launch_bounds__(kNormThreads) k_init_norm(const C* __restrict__ phi, long long n, double weight,
@@ -379,10 +378,8 @@ __global__ void __launch_bounds__(kNormThreads) k_init_norm(const C* __restrict_
   __threadfence();
   double tot = 0.0;
   for (unsigned b = 0; b < gridDim.x; ++b) tot += __ldcg(partials + b);
-  ctl->c = 1.0;
-  ctl->s = 0.0;
-  ctl->inv_np = 0.0;
-  ctl->inv_nrm = 1.0 / sqrt(weight * tot);
+  ctl->cc = num(1.0 / sqrt(weight * tot));
+  ctl->ss = num(0.0);
   ctl->retract = 1;
   *ticket = 0u;  // ready for the next reduction
 }

@@ -168,10 +168,6 @@ extern "C" gpe_status gpe_apply_H_noalloc(const gpe_problem* prob, const void* V
   }
   unsigned char* base = static_cast<unsigned char*>(g_scratch_addr[dev]);
 
-  // The reduction ticket must start at zero; the other contents are fully
-  // rewritten before they are read.
-  e = cudaMemsetAsync(base + kTicketOff, 0, sizeof(unsigned), st);
-  if (e != cudaSuccess) { set_err(err, err_len, cudaGetErrorString(e)); return GPE_ERR_CUDA; }
   if (mode)
     k_noalloc_tables<double><<<1, 256, 0, st>>>(reinterpret_cast<double*>(base + kTablesOff), prob->dim, n[0], n[1],
                                                  n[2], prob->L[0], prob->L[1], prob->L[2]);
@@ -188,6 +184,8 @@ extern "C" gpe_status gpe_apply_H_noalloc(const gpe_problem* prob, const void* V
     a.dim = prob->dim; a.nx = n[0]; a.ny = n[1]; a.nz = prob->dim == 3 ? n[2] : 1;
     a.axis = ax; a.M = n[ax];
     a.weight = weight; a.eta = prob->eta; a.omega = prob->omega;
+    a.eta_n = num(a.eta); a.omega_n = num(a.omega);
+    a.nomoments = 1;  // H phi as a plain operator: no reductions
     for (int i = 0; i < 3; ++i) {
       a.xi[i] = base + kTablesOff + (size_t)i * 4 * 512 * tsz;
       a.xc[i] = base + kTablesOff + ((size_t)i * 4 * 512 + 512) * tsz;
@@ -198,8 +196,6 @@ extern "C" gpe_status gpe_apply_H_noalloc(const gpe_problem* prob, const void* V
     a.f = f_dev;
     a.t = base + kFieldOff;
     a.ctl = reinterpret_cast<Ctl*>(base + kCtlOff);
-    a.partials = reinterpret_cast<double*>(base + kPartialsOff);
-    a.ticket = reinterpret_cast<unsigned*>(base + kTicketOff);
     if (ax == 0) {
       a.lpb = lpb;
       a.nblocks = (int)blocks_ax[0];

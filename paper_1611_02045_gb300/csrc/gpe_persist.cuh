@@ -64,9 +64,11 @@ __device__ __forceinline__ bool grid_sync(const PersistArgs& P) {
 }
 
 // Block partials -> barrier -> fixed-order total in every block (tot[] in
-// shared memory, FP64, valid in all threads on return).
-template <int K, unsigned MAXMASK>
+// shared memory, FP64, weighted, valid in all threads on return).
+template <int ROLE>
 __device__ __forceinline__ bool all_reduce(const PersistArgs& P, const Acc* acc, int& parity, double* tot) {
+  constexpr int K = Moments<ROLE>::K;
+  constexpr unsigned MAXMASK = Moments<ROLE>::MAX;
   __shared__ Acc red_sm[32 * kMaxMoments];
   Acc v[K];
 #pragma unroll
@@ -79,22 +81,9 @@ __device__ __forceinline__ bool all_reduce(const PersistArgs& P, const Acc* acc,
   }
   if (!grid_sync(P)) return false;
   Acc w[K];
-#pragma unroll
-  for (int k = 0; k < K; ++k) w[k] = Acc{0.0f, 0.0f};
-#pragma unroll 4
-  for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x) {
-    const float2* pb = reinterpret_cast<const float2*>(part + (size_t)b * kMaxMoments);
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const float2 x = __ldcg(pb + k);
-      w[k] = red_op<MAXMASK>(w[k], Acc{x.x, x.y}, k);
-    }
-  }
+  sum_partials<K, MAXMASK>(part, (int)gridDim.x, w);
   block_reduce<K, MAXMASK>(w, red_sm);
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) tot[k] = acc_to_double(w[k]);
-  }
+  totals<K, Moments<ROLE>::W>(w, P.hx.weight, tot);
   __syncthreads();
   parity ^= 1;
   return true;
@@ -125,7 +114,8 @@ template <int MODE, int M, int DIM>
 __global__ void __launch_bounds__(256) persist_solve(PersistArgs P) {
   extern __shared__ __align__(16) unsigned char smraw[];
   __shared__ Ctl S;
-  __shared__ double tot[kMaxMoments];
+  __shared__ double tot[3][kMaxMoments];  // per axis of the operator under way
+  const bool lead = threadIdx.x < (full_warp() ? 32 : 1);  // runs the scalar steps
   if (threadIdx.x == 0) S = *P.ctl;
   __syncthreads();
   const bool writer = blockIdx.x == 0;
@@ -139,34 +129,20 @@ __global__ void __launch_bounds__(256) persist_solve(PersistArgs P) {
     // ---- H phi_n (x pass folds in the retraction to phi_n) ----
     Scal sc = scal_of(&S, P.hx);
     x_phase<MODE, M, P_HX>(P.hx, sc, U, smraw, acc);
-    if (!(ok = all_reduce<6, 32u>(P, acc, parity, tot))) break;
-    if (threadIdx.x == 0)
-      for (int k = 0; k < 6; ++k) S.hsum[0][k] = tot[k];
+    if (!(ok = all_reduce<P_HX>(P, acc, parity, tot[0]))) break;
     s_phase<MODE, M, P_HMID>(P.hy, sc, U, smraw, acc);
-    if (!(ok = all_reduce<2, 0u>(P, acc, parity, tot))) break;
-    if (threadIdx.x == 0) {
-      S.hsum[1][0] = tot[0];
-      S.hsum[1][1] = tot[1];
-      if (DIM == 2) finalize_H(&S, F, writer);
-    }
+    if (!(ok = all_reduce<P_HMID>(P, acc, parity, tot[1]))) break;
     if constexpr (DIM == 3) {
       s_phase<MODE, M, P_HMID>(P.hz, sc, U, smraw, acc);
-      if (!(ok = all_reduce<2, 0u>(P, acc, parity, tot))) break;
-      if (threadIdx.x == 0) {
-        S.hsum[2][0] = tot[0];
-        S.hsum[2][1] = tot[1];
-        finalize_H(&S, F, writer);
-      }
+      if (!(ok = all_reduce<P_HMID>(P, acc, parity, tot[2]))) break;
     }
+    if (lead) finalize_H(&S, F, tot[0], tot[1], tot[2], writer);
     __syncthreads();
     // ---- residual, stopping rule, P_C r_n ----
     sc = scal_of(&S, P.c1);
     x_phase<MODE, M, P_C1>(P.c1, sc, U, smraw, acc);
-    if (!(ok = all_reduce<3, 1u>(P, acc, parity, tot))) break;
-    if (threadIdx.x == 0) {
-      const double t3[3] = {tot[0], tot[1], tot[2]};
-      finalize_C1(&S, F, t3, writer);
-    }
+    if (!(ok = all_reduce<P_C1>(P, acc, parity, tot[0]))) break;
+    if (lead) finalize_C1(&S, tot[0], writer);
     __syncthreads();
     if (S.done) break;
     if constexpr (DIM == 3) {
@@ -180,32 +156,20 @@ __global__ void __launch_bounds__(256) persist_solve(PersistArgs P) {
       if (!(ok = grid_sync(P))) break;
     }
     x_phase<MODE, M, P_C3>(P.c3, sc, U, smraw, acc);
-    if (!(ok = all_reduce<6, 0u>(P, acc, parity, tot))) break;
-    if (threadIdx.x == 0) {
-      const double t6[6] = {tot[0], tot[1], tot[2], tot[3], tot[4], tot[5]};
-      finalize_C3(&S, F, t6, writer);
-    }
+    if (!(ok = all_reduce<P_C3>(P, acc, parity, tot[0]))) break;
+    if (lead) finalize_C3(&S, tot[0], writer);
     __syncthreads();
     // ---- p_n and the step size ----
     sc = scal_of(&S, P.ax);
     x_phase<MODE, M, P_AX>(P.ax, sc, U, smraw, acc);
-    if (!(ok = all_reduce<9, 0u>(P, acc, parity, tot))) break;
-    if (threadIdx.x == 0)
-      for (int k = 0; k < 9; ++k) S.asum[0][k] = tot[k];
+    if (!(ok = all_reduce<P_AX>(P, acc, parity, tot[0]))) break;
     s_phase<MODE, M, P_AMID>(P.ay, sc, U, smraw, acc);
-    if (!(ok = all_reduce<1, 0u>(P, acc, parity, tot))) break;
-    if (threadIdx.x == 0) {
-      S.asum[1][1] = tot[0];
-      if (DIM == 2) finalize_A(&S, F, writer);
-    }
+    if (!(ok = all_reduce<P_AMID>(P, acc, parity, tot[1]))) break;
     if constexpr (DIM == 3) {
       s_phase<MODE, M, P_AMID>(P.az, sc, U, smraw, acc);
-      if (!(ok = all_reduce<1, 0u>(P, acc, parity, tot))) break;
-      if (threadIdx.x == 0) {
-        S.asum[2][1] = tot[0];
-        finalize_A(&S, F, writer);
-      }
+      if (!(ok = all_reduce<P_AMID>(P, acc, parity, tot[2]))) break;
     }
+    if (lead) finalize_A(&S, F, tot[0], tot[1][0], DIM == 3 ? tot[2][0] : 0.0, writer);
     __syncthreads();
   }
   if (threadIdx.x == 0) {
