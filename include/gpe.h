@@ -374,8 +374,9 @@ gpe_status gpe_apply_H_noalloc(const gpe_problem* prob, const void* V_dev, const
  * radix 8 then 8/4/2 stages for E = 8, radix-4 stages for E = 4), blocks of
  * `width` lines (x passes) or tiles of `width` adjacent x-columns (y, z
  * passes).  A plan (E, width) is kept per launch mode (0: complex64 passes,
- * 1: FP64 passes, 2: refinement passes) and axis; the defaults are E = 8 and
- * widths from a block-count heuristic.  Plans change the order of floating-
+ * 1: FP64 passes, 2: refinement passes) and axis; the defaults are E = 8, or
+ * E = 4 for FP64 and refinement passes on small grids, and widths from a
+ * block-count heuristic.  Plans change the order of floating-
  * point sums, not the method.  The paper has no counterpart (it runs serial
  * full-grid FFTs). */
 typedef struct {

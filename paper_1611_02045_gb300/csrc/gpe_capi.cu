@@ -24,7 +24,7 @@ using namespace gpe;
 
 namespace {
 
-constexpr int kTargetBlocks = 2 * 152;  // aim for >= 2 blocks per SM per pass
+constexpr int kTargetBlocks = 128;  // default plans: blocks wanted per pass (152 SMs)
 constexpr int kPlanMaxBlocks = 4096;    // reduction partials reserved for tuned plans
 
 struct PassPlan {
@@ -67,8 +67,7 @@ struct gpe_ctx {
   unsigned* ticket = nullptr;  // [0] reduction ticket, [1..3] blocks in each region of the partials
   double* log_dev = nullptr;
   int log_dev_cap = 0;
-  PassPlan plan[3];      // default plan per axis (E = 8, heuristic widths)
-  PassPlan mplan[3][3];  // plan used per launch mode [mode][axis] (the default, or the tuner's choice)
+  PassPlan mplan[3][3];  // plan used per launch mode [mode][axis] (plan_axis, or the tuner's choice)
   int partials_cap = 0;  // blocks the reduction partials buffer holds
   int hbatch_rows = 16;  // rows per CTA of its streaming form (plan mode 3 width: 16 or 32)
   int* hflow_ctr = nullptr;  // counters of gpe_apply_H_batch's dataflow form (zero between launches)
@@ -112,29 +111,44 @@ static bool is_device_ptr(const void* p) {
   return at.type == cudaMemoryTypeDevice || at.type == cudaMemoryTypeManaged;
 }
 
-static void plan_axis(gpe_ctx* c, int axis, int maxT, PassPlan& pl) {
+// Default plan of (mode, axis).
+//  * E values per thread: 8, or 4 where the threads are what is missing.  The FP64
+//    pipe takes one warp instruction per sub-partition every 64 cycles, so an FP64
+//    pass lasts as long as its busiest of 608 sub-partitions, and double-single
+//    passes are long instruction chains: up to 2^17 points (at most 512 warps at E =
+//    8) both run at E = 4, which halves each thread's work (256^2: FP64 178 -> 123
+//    us per iteration, refinement 113 -> 83; 512^2 FP64: no gain).  The refinement's
+//    x passes do at every size (128^3: 531 -> 486).  FP32 passes keep E = 8, which
+//    the TMA-fed kernels need.
+//  * width: the widest block up to the thread cap, halved while the axis has fewer
+//    than 128 blocks and the block more than one warp: blocks below a warp waste
+//    lanes, and every block costs a ticket and a partial (32^3 with blocks of 8
+//    threads: 158 us per complex64 iteration against 79 with these widths).
+static void plan_axis(const gpe_ctx* c, int mode, int axis, PassPlan& pl) {
   const int M = c->n[axis];
+  const bool few = c->N <= (1ll << 17);
+  pl.E = (M >= 32 && ((mode == 1 && few) || (mode == 2 && (few || axis == 0)))) ? 4 : 8;
   const int Tl = M / pl.E;
+  const int maxT = c->max_threads[1];  // the smaller (FP64) thread cap
   pl.M = M;
+  const long long per = axis == 0 ? 1 : c->n[0];  // columns per outer index
+  const long long outer = axis == 0 ? (long long)c->n[1] * (c->dim == 3 ? c->n[2] : 1)
+                                    : (axis == 1 ? (c->dim == 3 ? c->n[2] : 1) : c->n[1]);
+  int w = maxT / Tl;
+  if (w < 1) w = 1;
+  if (axis > 0 && w > 16) w = 16;
+  while (w > 1 && w > (axis == 0 ? outer : per)) w >>= 1;
+  auto blocks = [&](int v) { return axis == 0 ? outer / v : per / v * outer; };
+  const int least = axis == 0 ? 1 : (mode == 0 ? 4 : 2);  // strided tiles: 32-byte sectors
+  while (w > least && w * Tl > 32 && blocks(w) < kTargetBlocks) w >>= 1;
+  pl.nblocks = (int)blocks(w);
   if (axis == 0) {
-    const long long nlines = (long long)c->n[1] * (c->dim == 3 ? c->n[2] : 1);
-    int lpb = maxT / Tl;
-    if (lpb < 1) lpb = 1;
-    while (lpb > 1 && (lpb > nlines || nlines / lpb < kTargetBlocks)) lpb >>= 1;
-    pl.lpb = lpb;
-    pl.nblocks = (int)(nlines / lpb);
+    pl.lpb = w;
   } else {
-    const int nx = c->n[0];
-    const long long outer = (axis == 1) ? (c->dim == 3 ? c->n[2] : 1) : c->n[1];
-    int tx = 16;
-    if (tx > nx) tx = nx;
-    while (tx > 1 && tx * Tl > maxT) tx >>= 1;
-    while (tx > 4 && (long long)(nx / tx) * outer < kTargetBlocks) tx >>= 1;
-    pl.tx = tx;
-    pl.ntx = nx / tx;
-    pl.nblocks = (int)((long long)pl.ntx * outer);
-    pl.stride = (axis == 1) ? nx : (long long)nx * c->n[1];
-    pl.outer_stride = (axis == 1) ? (long long)nx * c->n[1] : nx;
+    pl.tx = w;
+    pl.ntx = c->n[0] / w;
+    pl.stride = (axis == 1) ? c->n[0] : (long long)c->n[0] * c->n[1];
+    pl.outer_stride = (axis == 1) ? (long long)c->n[0] * c->n[1] : c->n[0];
   }
 }
 
@@ -346,10 +360,10 @@ extern "C" gpe_status gpe_create(const gpe_problem* prob, const double* V, void*
 
   int maxblocks = 1;
   for (int ax = 0; ax < c->dim; ++ax) {
-    // plan with the smaller (double) thread cap so one plan serves both precisions
-    plan_axis(c, ax, c->max_threads[1], c->plan[ax]);
-    if (c->plan[ax].nblocks > maxblocks) maxblocks = c->plan[ax].nblocks;
-    for (int m = 0; m < 3; ++m) c->mplan[m][ax] = c->plan[ax];
+    for (int m = 0; m < 3; ++m) {
+      plan_axis(c, m, ax, c->mplan[m][ax]);
+      if (c->mplan[m][ax].nblocks > maxblocks) maxblocks = c->mplan[m][ax].nblocks;
+    }
   }
   c->partials_cap = maxblocks > kPlanMaxBlocks ? maxblocks : kPlanMaxBlocks;  // room for tuned plans
   if (cudaMalloc(&c->ctl_solve, sizeof(Ctl)) != cudaSuccess || cudaMalloc(&c->ctl_api, sizeof(Ctl)) != cudaSuccess ||
