@@ -126,24 +126,18 @@ __global__ void __launch_bounds__(512) pass_s_tma(PassArgs a, const __grid_const
 #pragma unroll
       for (int q = 0; q < E; ++q) tv[q] = in0[tile + (t + q * Tl) * tx + c];
       line_dft<M, E, -1>(v, ex, si, t, tw);
-      const T x = (a.axis == 1) ? tab<T>(a.xc[0])[ix] : T(0);
-      const T rx = (a.axis == 1) ? -x : T(0);  // rotation symbol -omega x mu (y); none for z
-      T akin = 0, arot = 0;
-#pragma unroll
-      for (int q = 0; q < E; ++q) {
-        const T k = xia[t + q * Tl];
-        const T mk = T(0.5) * k * k, kr = rx * k;
-        const T a2 = v[q].x * v[q].x + v[q].y * v[q].y;
-        akin += mk * a2;
-        arot += kr * a2;
-        v[q] = cscale(v[q], (mk + om * kr) * invM);
+      const T rx = (a.axis == 1) ? -tab<T>(a.xc[0])[ix] : T(0);  // rotation symbol -omega x mu (y); none for z
+      if (!a.nomoments) {
+        T s1, s2;
+        symbol_sums<E>(v, xia, t, Tl, s1, s2);
+        acc[0] = acc_add(acc[0], acc_from(T(0.5) * s2 * invM));
+        acc[1] = acc_add(acc[1], acc_from(rx * s1 * invM));
       }
+      apply_symbol<E>(v, xia, t, Tl, T(0.5) * invM, om * rx * invM);
       line_dft<M, E, +1>(v, ex, si, t, tw);
       C* __restrict__ dst = static_cast<C*>(a.out ? a.out : a.t);  // API: the final pass writes the caller's buffer
 #pragma unroll
       for (int q = 0; q < E; ++q) dst[base + (t + q * Tl) * a.stride] = cadd(tv[q], v[q]);
-      acc[0] = acc_add(acc[0], acc_from(akin * invM));
-      acc[1] = acc_add(acc[1], acc_from(arot * invM));
     } else if constexpr (ROLE == P_CFWD || ROLE == P_CINV || ROLE == P_CCORE) {
       if constexpr (ROLE == P_CINV) {
         line_dft<M, E, +1>(v, ex, si, t, tw);
@@ -181,7 +175,7 @@ __global__ void __launch_bounds__(512) pass_s_tma(PassArgs a, const __grid_const
 #pragma unroll
       for (int q = 0; q < E; ++q) {
         const T k = xia[t + q * Tl];
-        akr += (T(0.5) * k * k + rs * k) * (v[q].x * v[q].x + v[q].y * v[q].y);
+        akr += k * (T(0.5) * k + rs) * (v[q].x * v[q].x + v[q].y * v[q].y);
       }
       acc[0] = acc_add(acc[0], acc_from(akr * invM));
     }
@@ -288,35 +282,36 @@ __global__ void __launch_bounds__(512) pass_hx_bulk(PassArgs a, int second) {
     }
     line_dft<M, E, -1, W>(v, sm, si, t, tw);
     const T y = tab<T>(a.xc[1])[iy];
-    T akin = 0, arot = 0;  // arot: the rotation symbol without omega (omega is applied in finalize_H)
-#pragma unroll
-    for (int q = 0; q < E; ++q) {
-      const T k = xi[t + q * Tl];
-      const T mk = T(0.5) * k * k, kr = y * k;
-      const T a2 = v[q].x * v[q].x + v[q].y * v[q].y;
-      akin += mk * a2;
-      arot += kr * a2;
-      v[q] = cscale(v[q], (mk + om * kr) * invM);
+    if (!a.nomoments) {  // the rotation symbol without omega (applied in finalize_H)
+      T s1, s2;
+      symbol_sums<E>(v, xi, t, Tl, s1, s2);
+      acc[0] = acc_add(acc[0], acc_from(T(0.5) * s2 * invM));
+      acc[1] = acc_add(acc[1], acc_from(y * s1 * invM));
     }
+    apply_symbol<E>(v, xi, t, Tl, T(0.5) * invM, om * y * invM);
     line_dft<M, E, +1, W>(v, sm, si, t, tw);
-    T apot = 0, au2 = 0, an2 = 0, umax = 0;
 #pragma unroll
     for (int q = 0; q < E; ++q) {
       const T uu = ph[q].x * ph[q].x + ph[q].y * ph[q].y;
       const T m = vv[q] + eta * uu;
       const C fq = (second == 1) ? secs[q * Tl] : ph[q];  // the operand f (API call with f != phi)
       tout[base + q * Tl] = make_float2(v[q].x + m * fq.x, v[q].y + m * fq.y);
-      apot += vv[q] * uu;
-      au2 += uu * uu;
-      an2 += uu;
-      umax = fmaxf(umax, uu);
     }
-    acc[0] = acc_add(acc[0], acc_from(akin * invM));
-    acc[1] = acc_add(acc[1], acc_from(arot * invM));
-    acc[2] = acc_add(acc[2], acc_from(apot));
-    acc[3] = acc_add(acc[3], acc_from(au2));
-    acc[4] = acc_add(acc[4], acc_from(an2));
-    acc[5] = acc_max(acc[5], acc_from(umax));
+    if (!a.nomoments) {
+      T apot = 0, au2 = 0, an2 = 0, umax = 0;
+#pragma unroll
+      for (int q = 0; q < E; ++q) {
+        const T uu = ph[q].x * ph[q].x + ph[q].y * ph[q].y;
+        apot += vv[q] * uu;
+        au2 += uu * uu;
+        an2 += uu;
+        umax = fmaxf(umax, uu);
+      }
+      acc[2] = acc_add(acc[2], acc_from(apot));
+      acc[3] = acc_add(acc[3], acc_from(au2));
+      acc[4] = acc_add(acc[4], acc_from(an2));
+      acc[5] = acc_max(acc[5], acc_from(umax));
+    }
     __syncthreads();  // stage s is read by every thread before it is refilled
   }
   reduce_and_finish<P_HX>(a, acc);

@@ -524,6 +524,14 @@ __device__ __forceinline__ bool pc_core(int k) { return !(k == 2 || k == 5); }
 template <typename T> __device__ __forceinline__ T pv_factor(T den, int code) {
   return code == 0 ? T(1) : (code == 2 ? T(1) / den : T(1) / sqrt(den));
 }
+// FP64: one reciprocal square root instead of a square root and a division.
+template <> __device__ __forceinline__ double pv_factor<double>(double den, int code) {
+  return code == 0 ? 1.0 : (code == 2 ? __drcp_rn(den) : rsqrt(den));
+}
+// p / den for a power of two p: FP64 takes the (correctly rounded) reciprocal,
+// whose scaling is exact, in place of the longer division.
+template <typename T> __device__ __forceinline__ T over(T p, T den) { return p / den; }
+template <> __device__ __forceinline__ double over<double>(double p, double den) { return p * __drcp_rn(den); }
 
 __device__ __forceinline__ Scal scal_of(const Ctl* c, const PassArgs& a) {
   Scal S;
@@ -542,6 +550,29 @@ __device__ __forceinline__ Scal scal_of(const Ctl* c, const PassArgs& a) {
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ const T* tab(const void* p) { return static_cast<const T*>(p); }
+
+// s1 = sum k |v|^2, s2 = sum k^2 |v|^2 over this thread's modes (k = xi[t + q Tl]):
+// Parseval's sums of the rotation and (twice) the kinetic symbol.
+template <int E, typename T, typename C>
+__device__ __forceinline__ void symbol_sums(const C (&v)[E], const T* __restrict__ xi, int t, int Tl, T& s1, T& s2) {
+  s1 = T(0);
+  s2 = T(0);
+#pragma unroll
+  for (int q = 0; q < E; ++q) {
+    const T k = xi[t + q * Tl], ka = k * (v[q].x * v[q].x + v[q].y * v[q].y);
+    s1 += ka;
+    s2 += k * ka;
+  }
+}
+// v *= k (h k + c): the symbol (1/2 k^2 + r k) / M with h = 1/(2M), c = r / M.
+template <int E, typename T, typename C>
+__device__ __forceinline__ void apply_symbol(C (&v)[E], const T* __restrict__ xi, int t, int Tl, T h, T c) {
+#pragma unroll
+  for (int q = 0; q < E; ++q) {
+    const T k = xi[t + q * Tl];
+    v[q] = cscale(v[q], k * (h * k + c));
+  }
+}
 
 // ---------------------------------------------------------------------------
 // Contiguous (x) passes.  Block = lpb lines x Tl threads; tid = t + Tl*l.
@@ -634,20 +665,16 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
     }
     line_dft<M, E, -1, W>(v, sm, si, t, tw);
     const TF y = tab<TF>(a.xc[1])[iy];
-    const TF om = num_as<TF>(a.omega_n);
-    TF akin = 0, arot = 0;  // arot: the rotation symbol without omega (omega is applied in finalize_H)
-#pragma unroll
-    for (int q = 0; q < E; ++q) {
-      const TF k = xi[t + q * Tl];
-      const TF mk = TF(0.5) * k * k, kr = y * k;
-      const TF a2 = v[q].x * v[q].x + v[q].y * v[q].y;
-      akin += mk * a2; arot += kr * a2;
-      v[q] = cscale(v[q], (mk + om * kr) * invM);
+    if (!a.nomoments) {  // uniform; the rotation symbol without omega (applied in finalize_H)
+      TF s1, s2;
+      symbol_sums<E>(v, xi, t, Tl, s1, s2);
+      acc[0] = acc_add(acc[0], acc_from(TF(0.5) * s2 * invM));
+      acc[1] = acc_add(acc[1], acc_from(y * s1 * invM));
     }
+    apply_symbol<E>(v, xi, t, Tl, TF(0.5) * invM, num_as<TF>(a.omega_n) * y * invM);
     line_dft<M, E, +1, W>(v, sm, si, t, tw);
     CS* __restrict__ tout = static_cast<CS*>(a.t);
     const TS eta = num_as<TS>(a.eta_n);
-    TS apot = 0, au2 = 0, an2 = 0, umax = 0;
 #pragma unroll
     for (int q = 0; q < E; ++q) {
       const long long g = base + t + q * Tl;
@@ -655,14 +682,20 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
       const TS m = vv[q] + eta * u;
       const CS fq = (a.f && !a.solver) ? f[g] : ph[q];  // the operand f (re-read in API mode)
       tout[g] = cmk<CS>(TS(v[q].x) + m * fq.x, TS(v[q].y) + m * fq.y);
-      apot += vv[q] * u; au2 += u * u; an2 += u; umax = fmax(umax, u);
     }
-    acc[0] = acc_add(acc[0], acc_from(akin * invM));
-    acc[1] = acc_add(acc[1], acc_from(arot * invM));
-    acc[2] = acc_add(acc[2], acc_from(apot));
-    acc[3] = acc_add(acc[3], acc_from(au2));
-    acc[4] = acc_add(acc[4], acc_from(an2));
-    acc[5] = acc_max(acc[5], acc_from(umax));
+    if (!a.nomoments) {
+      TS apot = 0, au2 = 0, an2 = 0, umax = 0;
+#pragma unroll
+      for (int q = 0; q < E; ++q) {
+        const TS u = ph[q].x * ph[q].x + ph[q].y * ph[q].y;
+        apot += vv[q] * u; au2 += u * u; an2 += u;
+        if constexpr (sizeof(TS) == 4) umax = fmax(umax, u);  // read by the complex64 phase's switch rule only
+      }
+      acc[2] = acc_add(acc[2], acc_from(apot));
+      acc[3] = acc_add(acc[3], acc_from(au2));
+      acc[4] = acc_add(acc[4], acc_from(an2));
+      acc[5] = acc_max(acc[5], acc_from(umax));
+    }
   } else if constexpr (ROLE == P_C1) {
     // ---- s = FFT_x[P_V^{1/2} r], r = H phi - lambda phi (solver) or r_in (API) ----
     const CS* __restrict__ phi = static_cast<const CS*>(a.phi);
@@ -702,15 +735,18 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
     const TS alpha = num_as<TS>(S.alpha);
     const TS eta = num_as<TS>(a.eta_n);
     if (!a.solver) {
-      line_dft<M, E, +1, W>(v, sm, si, t, tw);
-      CD* __restrict__ out = static_cast<CD*>(a.out);
+      TS den[E];  // loaded before the transform, which hides the latency
 #pragma unroll
       for (int q = 0; q < E; ++q) {
         const long long g = base + t + q * Tl;
         const CS ph = phi[g];
-        const TS den = alpha + V[g] + eta * (ph.x * ph.x + ph.y * ph.y);
-        out[g] = cconv<TD>(cscale(cconv<TS>(v[q]), pv_factor(den, pc_post(S.pc))));
+        den[q] = alpha + V[g] + eta * (ph.x * ph.x + ph.y * ph.y);
       }
+      line_dft<M, E, +1, W>(v, sm, si, t, tw);
+      CD* __restrict__ out = static_cast<CD*>(a.out);
+#pragma unroll
+      for (int q = 0; q < E; ++q)
+        out[base + t + q * Tl] = cconv<TD>(cscale(cconv<TS>(v[q]), pv_factor(den[q], pc_post(S.pc))));
       return;
     }
     // every operand of the epilogue is loaded before the transform, so the
@@ -783,12 +819,12 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
     for (int q = 0; q < E; ++q) pbuf[base + t + q * Tl] = cconv<TD>(v[q]);
     line_dft<M, E, -1, W>(v, sm, si, t, tw);
     const TF y = tab<TF>(a.xc[1])[iy];
-    const TF om = num_as<TF>(a.omega_n);
+    const TF oy = num_as<TF>(a.omega_n) * y;
     TF akr = 0;
 #pragma unroll
     for (int q = 0; q < E; ++q) {
       const TF k = xi[t + q * Tl];
-      akr += (TF(0.5) * k * k + om * y * k) * (v[q].x * v[q].x + v[q].y * v[q].y);
+      akr += k * (TF(0.5) * k + oy) * (v[q].x * v[q].x + v[q].y * v[q].y);
     }
     acc[0] = acc_add(acc[0], acc_from(aR));
     acc[1] = acc_add(acc_add(acc[1], acc_from(aV)), acc_from(akr * invM));
@@ -834,24 +870,18 @@ __device__ __forceinline__ void sunit(const PassArgs& a, const Scal& S, long lon
     }
     if (S.done) return;
     line_dft<M, E, -1>(v, sm, si, t, tw);
-    const T om = num_as<T>(a.omega_n);
-    const T x = (a.axis == 1) ? tab<T>(a.xc[0])[ix] : T(0);
-    const T rx = (a.axis == 1) ? -x : T(0);  // rotation symbol -omega x mu (y), omega applied below; none for z
-    T akin = 0, arot = 0;
-#pragma unroll
-    for (int q = 0; q < E; ++q) {
-      const T k = xia[t + q * Tl];
-      const T mk = T(0.5) * k * k, kr = rx * k;
-      const T a2 = v[q].x * v[q].x + v[q].y * v[q].y;
-      akin += mk * a2; arot += kr * a2;
-      v[q] = cscale(v[q], (mk + om * kr) * invM);
+    const T rx = (a.axis == 1) ? -tab<T>(a.xc[0])[ix] : T(0);  // rotation symbol -omega x mu (y); none for z
+    if (!a.nomoments) {
+      T s1, s2;
+      symbol_sums<E>(v, xia, t, Tl, s1, s2);
+      acc[0] = acc_add(acc[0], acc_from(T(0.5) * s2 * invM));
+      acc[1] = acc_add(acc[1], acc_from(rx * s1 * invM));
     }
+    apply_symbol<E>(v, xia, t, Tl, T(0.5) * invM, num_as<T>(a.omega_n) * rx * invM);
     line_dft<M, E, +1>(v, sm, si, t, tw);
     C* __restrict__ dst = static_cast<C*>(a.out ? a.out : a.t);  // API: final pass writes the caller's buffer
 #pragma unroll
     for (int q = 0; q < E; ++q) dst[base + (t + q * Tl) * st] = cadd(tv[q], v[q]);
-    acc[0] = acc_add(acc[0], acc_from(akin * invM));
-    acc[1] = acc_add(acc[1], acc_from(arot * invM));
   } else if constexpr (ROLE == P_CFWD || ROLE == P_CINV || ROLE == P_CCORE) {
     C* __restrict__ sb = static_cast<C*>(a.s);
 #pragma unroll
@@ -878,7 +908,7 @@ __device__ __forceinline__ void sunit(const PassArgs& a, const Scal& S, long lon
       for (int q = 0; q < E; ++q) {
         const T k = xia[t + q * Tl];
         const T den = alpha + T(0.5) * (kx * kx + kother + k * k);
-        v[q] = cscale(v[q], core ? invN / den : invN);
+        v[q] = cscale(v[q], core ? over(invN, den) : invN);
       }
       line_dft<M, E, +1>(v, sm, si, t, tw);
     }
@@ -897,7 +927,7 @@ __device__ __forceinline__ void sunit(const PassArgs& a, const Scal& S, long lon
 #pragma unroll
     for (int q = 0; q < E; ++q) {
       const T k = xia[t + q * Tl];
-      akr += (T(0.5) * k * k + rs * k) * (v[q].x * v[q].x + v[q].y * v[q].y);
+      akr += k * (T(0.5) * k + rs) * (v[q].x * v[q].x + v[q].y * v[q].y);
     }
     acc[0] = acc_add(acc[0], acc_from(akr * invM));
   }
