@@ -14,7 +14,11 @@ namespace gpe {
 
 namespace {
 
-constexpr int kDotThreads = 256;
+// Blocks of one warp per SM sub-partition: an FP64 instruction holds its
+// sub-partition's pipe for 64 cycles per warp, so these kernels last as long as
+// the warps' FP64 chains on the busiest sub-partition (256^2: 512 warps of four
+// points on 608 sub-partitions).
+constexpr int kDotThreads = 128;
 
 template <typename C> struct Real;
 template <> struct Real<float2> { using type = float; };
@@ -25,53 +29,151 @@ __device__ __forceinline__ double2 dconj_mul(double ax, double ay, double bx, do
   return make_double2(ax * bx + ay * by, ax * by - ay * bx);
 }
 
-// Block sum of NV doubles (shuffle tree within warps, then warp 0 over the
-// warp results; fixed order), written to partials[blockIdx.x * NV + j].
-template <int NV>
-__device__ __forceinline__ void block_sum_store(double (&v)[NV], double* __restrict__ partials) {
-  __shared__ double sm[kDotThreads / 32][NV];
+// Sums over a warp of up to eight values at once: each of the first three steps
+// halves the values a lane keeps as well as the lanes, 9 additions instead of 5
+// per value.  Lane l returns the total of value 4 (l/16 & 1) + 2 (l/8 & 1) + (l/4 & 1).
+__device__ __forceinline__ double warp_sum8(const double (&v)[8]) {
+  const int l = threadIdx.x & 31;
+  const bool b4 = l & 16, b3 = l & 8, b2 = l & 4;
+  double w[4], u[2];
 #pragma unroll
-  for (int j = 0; j < NV; ++j)
-    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0)
+  for (int j = 0; j < 4; ++j)
+    w[j] = (b4 ? v[4 + j] : v[j]) + __shfl_xor_sync(0xffffffffu, b4 ? v[j] : v[4 + j], 16);
 #pragma unroll
-    for (int j = 0; j < NV; ++j) sm[warp][j] = v[j];
+  for (int j = 0; j < 2; ++j) u[j] = (b3 ? w[2 + j] : w[j]) + __shfl_xor_sync(0xffffffffu, b3 ? w[j] : w[2 + j], 8);
+  double x = (b2 ? u[1] : u[0]) + __shfl_xor_sync(0xffffffffu, b2 ? u[0] : u[1], 4);
+  x += __shfl_xor_sync(0xffffffffu, x, 2);
+  x += __shfl_xor_sync(0xffffffffu, x, 1);
+  return x;
+}
+
+// Block totals (fixed order): in warp 0, lane l returns the total of value l mod 8.
+__device__ __forceinline__ double block_sum8(const double (&v)[8], double (*sm)[8]) {
+  constexpr int NW = kDotThreads / 32;
+  static_assert(NW == 4, "four warps: the last two steps sum over lane bits 3 and 4");
+  const int l = threadIdx.x & 31;
+  const double x = warp_sum8(v);
+  if ((l & 3) == 0) sm[threadIdx.x >> 5][4 * (l >> 4) + 2 * ((l >> 3) & 1) + ((l >> 2) & 1)] = x;
   __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int j = 0; j < NV; ++j) {
-      double x = lane < kDotThreads / 32 ? sm[lane][j] : 0.0;
-      for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-      if (lane == 0) partials[(size_t)blockIdx.x * NV + j] = x;
+  double t = 0.0;
+  if (threadIdx.x < 32) {
+    t = sm[l >> 3][l & 7];
+    t += __shfl_xor_sync(0xffffffffu, t, 8);
+    t += __shfl_xor_sync(0xffffffffu, t, 16);
+  }
+  return t;
+}
+
+// The scalar step `stage` from the weighted totals t (all lanes of warp 0 hold
+// them; lane 0 writes).
+__device__ __forceinline__ void adj_scalar_step(int stage, const double (&t)[6], AdjScalars* __restrict__ S) {
+  if (threadIdx.x != 0 || S->stop) return;  // stop: the solve has ended; later kernels of the last round change nothing
+  switch (stage) {
+    case ADJ_PROJ:  // t = <phi, h>
+      S->c_re = t[0]; S->c_im = t[1];
+      break;
+    case ADJ_BB:  // t = ||r0||^2
+      S->bb = t[0]; S->rr = t[0];
+      if (!isfinite(t[0])) { S->bad = 3; S->stop = 1; }
+      else if (t[0] == 0.0) S->stop = 1;  // P g = 0: z = 0
+      break;
+    case ADJ_PQ: {  // t = <phi, q>, <p, q>, <p, phi>;  Re<p, q - c phi>
+      S->c_re = t[0]; S->c_im = t[1];
+      // <p, c phi> = c <p, phi>
+      const double pq = t[2] - (t[0] * t[4] - t[1] * t[5]);
+      S->pq = pq;
+      if (!(pq > 0.0) || !isfinite(pq)) { S->bad = 1; S->stop = 1; }  // K not positive on the tangent space
+      else S->a = S->ry / pq;
+      break;
     }
+    case ADJ_RR:  // t = ||r||^2
+      S->rr = t[0];
+      S->iters += 1;
+      if (!isfinite(t[0])) { S->bad = 3; S->stop = 1; }
+      else if (t[0] <= S->tol2 * S->bb) S->stop = 1;  // ||r|| <= tol ||P g||
+      break;
+    case ADJ_RY:        // t = <phi, y>, <r, y>, <r, phi>;  Re<r, y - c phi>
+    case ADJ_RY_FIRST: {
+      S->c_re = t[0]; S->c_im = t[1];
+      const double ry = t[2] - (t[0] * t[4] - t[1] * t[5]);
+      S->beta = (stage == ADJ_RY_FIRST) ? 0.0 : ry / S->ry;
+      if (!(ry > 0.0) || !isfinite(ry)) { S->bad = 2; S->stop = 1; }  // preconditioner not positive
+      S->ry = ry;
+      break;
+    }
+    default:
+      break;
   }
 }
 
-// Up to three complex inner products sum conj(x_j) y_j (x_j null: skipped).
+// Sum over the grid in a fixed order: block totals to red.partials, and the last
+// block to arrive sums them and runs the scalar step, so that a reduction needs
+// no kernel of its own (one that summed 1024 slots on one SM took 17.6 us).
+struct AdjRed {
+  double* partials;  // [blocks][8]
+  unsigned* ticket;  // zero on entry, zero on return
+  double weight;
+  int stage;
+  AdjScalars* S;
+};
+__device__ __forceinline__ void adj_reduce(const double (&v)[8], const AdjRed& red) {
+  __shared__ double sm[kDotThreads / 32][8];
+  __shared__ int s_last;
+  double t = block_sum8(v, sm);
+  if (threadIdx.x < 8) red.partials[(size_t)blockIdx.x * 8 + threadIdx.x] = t;
+  if (threadIdx.x < 32) {
+    __threadfence();
+    __syncwarp();
+    if (threadIdx.x == 0) s_last = (atomicAdd(red.ticket, 1u) == gridDim.x - 1) ? 1 : 0;
+  }
+  __syncthreads();
+  if (!s_last) return;
+  __threadfence();
+  double w[8];
+#pragma unroll
+  for (int j = 0; j < 8; ++j) w[j] = 0.0;
+  for (unsigned b = threadIdx.x; b < gridDim.x; b += kDotThreads) {
+    const double2* pb = reinterpret_cast<const double2*>(red.partials + (size_t)b * 8);
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      const double2 x = __ldcg(pb + j);
+      w[2 * j] += x.x;
+      w[2 * j + 1] += x.y;
+    }
+  }
+  t = block_sum8(w, sm) * red.weight;
+  if (threadIdx.x >= 32) return;
+  double tot[6];
+#pragma unroll
+  for (int j = 0; j < 6; ++j) tot[j] = __shfl_sync(0xffffffffu, t, j);
+  adj_scalar_step(red.stage, tot, red.S);
+  if (threadIdx.x == 0) *red.ticket = 0u;
+}
+
+// Up to three inner products sum conj(x_j) y_j (x_j null: skipped; the real part of the second).
 template <typename C>
 __global__ void __launch_bounds__(kDotThreads) k_dots(const C* __restrict__ x0, const C* __restrict__ y0,
                                                       const C* __restrict__ x1, const C* __restrict__ y1,
                                                       const C* __restrict__ x2, const C* __restrict__ y2, long long n,
-                                                      double* __restrict__ partials) {
-  double v[6] = {0, 0, 0, 0, 0, 0};
+                                                      AdjRed red) {
+  double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     if (x0) { const C a = x0[i], b = y0[i]; const double2 d = dconj_mul(a.x, a.y, b.x, b.y); v[0] += d.x; v[1] += d.y; }
-    if (x1) { const C a = x1[i], b = y1[i]; const double2 d = dconj_mul(a.x, a.y, b.x, b.y); v[2] += d.x; v[3] += d.y; }
+    if (x1) { const C a = x1[i], b = y1[i]; v[2] += (double)a.x * b.x + (double)a.y * b.y; }  // real part
     if (x2) { const C a = x2[i], b = y2[i]; const double2 d = dconj_mul(a.x, a.y, b.x, b.y); v[4] += d.x; v[5] += d.y; }
   }
-  block_sum_store<6>(v, partials);
+  adj_reduce(v, red);
 }
 
 // q <- q + eta |phi|^2 p + eta phi^2 conj(p) - lam p  (q holds H_phi p on entry),
-// then the sums <phi, q>, <p, q>, <p, phi>.
+// then the sums <phi, q>, Re<p, q>, <p, phi>.
 template <typename C>
 __global__ void __launch_bounds__(kDotThreads) k_hess_epi(const C* __restrict__ phi, const C* __restrict__ p,
                                                           C* __restrict__ q, long long n, double eta, double lam,
-                                                          double* __restrict__ partials) {
+                                                          AdjRed red) {
   using R = typename Real<C>::type;
   const R e = R(eta), l = R(lam);
-  double v[6] = {0, 0, 0, 0, 0, 0};
+  double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const C f = phi[i], d = p[i];
     C h = q[i];
@@ -83,21 +185,22 @@ __global__ void __launch_bounds__(kDotThreads) k_hess_epi(const C* __restrict__ 
     h.y += e * (u * d.y + cy) - l * d.y;
     q[i] = h;
     double2 t = dconj_mul(f.x, f.y, h.x, h.y); v[0] += t.x; v[1] += t.y;
-    t = dconj_mul(d.x, d.y, h.x, h.y); v[2] += t.x; v[3] += t.y;
+    v[2] += (double)d.x * h.x + (double)d.y * h.y;
     t = dconj_mul(d.x, d.y, f.x, f.y); v[4] += t.x; v[5] += t.y;
   }
-  block_sum_store<6>(v, partials);
+  adj_reduce(v, red);
 }
 
 // z += a p; r -= a (q - c phi); and the sum |r|^2.
 template <typename C>
 __global__ void __launch_bounds__(kDotThreads) k_step(C* __restrict__ z, C* __restrict__ r, const C* __restrict__ p,
                                                       const C* __restrict__ q, const C* __restrict__ phi, long long n,
-                                                      const AdjScalars* __restrict__ S, double* __restrict__ partials) {
+                                                      AdjRed red) {
   using R = typename Real<C>::type;
+  const AdjScalars* S = red.S;
   if (S->stop) return;  // converged or broken down: leave z and r as they are
   const R a = R(S->a), cr = R(S->c_re), ci = R(S->c_im);
-  double v[2] = {0, 0};
+  double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
     const C d = p[i], h = q[i], f = phi[i];
     C zz = z[i], rr = r[i];
@@ -107,7 +210,7 @@ __global__ void __launch_bounds__(kDotThreads) k_step(C* __restrict__ z, C* __re
     z[i] = zz; r[i] = rr;
     v[0] += (double)rr.x * rr.x + (double)rr.y * rr.y;
   }
-  block_sum_store<2>(v, partials);
+  adj_reduce(v, red);
 }
 
 // h_out = h_in - c phi (c complex from S), h_out may alias h_in.
@@ -140,64 +243,6 @@ __global__ void k_dir(C* __restrict__ p, const C* __restrict__ y, const C* __res
     o.y = h.y - (cr * f.y + ci * f.x);
     if (keep) { const C q = p[i]; o.x += b * q.x; o.y += b * q.y; }
     p[i] = o;
-  }
-}
-
-// Fixed-order sum of the block partials (NV per block), then the scalar step.
-__global__ void k_finish(const double* __restrict__ partials, int nblk, int nv, double weight, int stage,
-                         AdjScalars* __restrict__ S) {
-  __shared__ double sm[32][6];
-  double v[6] = {0, 0, 0, 0, 0, 0};
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x)
-    for (int j = 0; j < nv; ++j) v[j] += partials[(size_t)b * nv + j];
-  for (int j = 0; j < 6; ++j)
-    for (int o = 16; o > 0; o >>= 1) v[j] += __shfl_xor_sync(0xffffffffu, v[j], o);
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (lane == 0)
-    for (int j = 0; j < 6; ++j) sm[warp][j] = v[j];
-  __syncthreads();
-  if (threadIdx.x != 0) return;
-  double t[6] = {0, 0, 0, 0, 0, 0};
-  for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
-    for (int j = 0; j < 6; ++j) t[j] += sm[w][j];
-  for (int j = 0; j < 6; ++j) t[j] *= weight;  // weighted inner products
-  if (S->stop) return;  // the solve has ended; later kernels of the last round change nothing
-  switch (stage) {
-    case ADJ_PROJ:  // t = <phi, h>
-      S->c_re = t[0]; S->c_im = t[1];
-      break;
-    case ADJ_BB:  // t = ||r0||^2
-      S->bb = t[0]; S->rr = t[0];
-      if (!isfinite(t[0])) { S->bad = 3; S->stop = 1; }
-      else if (t[0] == 0.0) S->stop = 1;  // P g = 0: z = 0
-      break;
-    case ADJ_PQ: {  // t = <phi, q>, <p, q>, <p, phi>;  Re<p, q - c phi>
-      S->c_re = t[0]; S->c_im = t[1];
-      // <p, c phi> = c <p, phi>
-      const double cpr = t[0] * t[4] - t[1] * t[5];
-      S->pq = t[2] - cpr;
-      if (!(S->pq > 0.0) || !isfinite(S->pq)) { S->bad = 1; S->stop = 1; }  // K not positive on the tangent space
-      else S->a = S->ry / S->pq;
-      break;
-    }
-    case ADJ_RR:  // t = ||r||^2
-      S->rr = t[0];
-      S->iters += 1;
-      if (!isfinite(t[0])) { S->bad = 3; S->stop = 1; }
-      else if (t[0] <= S->tol2 * S->bb) S->stop = 1;  // ||r|| <= tol ||P g||
-      break;
-    case ADJ_RY:        // t = <phi, y>, <r, y>, <r, phi>;  Re<r, y - c phi>
-    case ADJ_RY_FIRST: {
-      S->c_re = t[0]; S->c_im = t[1];
-      const double crp = t[0] * t[4] - t[1] * t[5];
-      const double ry = t[2] - crp;
-      S->beta = (stage == ADJ_RY_FIRST) ? 0.0 : ry / S->ry;
-      if (!(ry > 0.0) || !isfinite(ry)) { S->bad = 2; S->stop = 1; }  // preconditioner not positive
-      S->ry = ry;
-      break;
-    }
-    default:
-      break;
   }
 }
 
@@ -237,42 +282,39 @@ int grid_of(long long n, int max_blocks) {
 }  // namespace
 
 cudaError_t adj_dots(int prec, const void* x0, const void* y0, const void* x1, const void* y1, const void* x2,
-                     const void* y2, long long n, double weight, int stage, AdjScalars* S, double* partials,
-                     int max_blocks, cudaStream_t st) {
-  const int g = grid_of(n, max_blocks);
+                     const void* y2, long long n, double weight, int stage, const AdjWork& w, cudaStream_t st) {
+  const int g = grid_of(n, kAdjMaxBlocks);
+  const AdjRed red = {w.partials, w.ticket, weight, stage, w.S};
   if (prec == 1)
     k_dots<double2><<<g, kDotThreads, 0, st>>>((const double2*)x0, (const double2*)y0, (const double2*)x1,
-                                               (const double2*)y1, (const double2*)x2, (const double2*)y2, n, partials);
+                                               (const double2*)y1, (const double2*)x2, (const double2*)y2, n, red);
   else
     k_dots<float2><<<g, kDotThreads, 0, st>>>((const float2*)x0, (const float2*)y0, (const float2*)x1,
-                                              (const float2*)y1, (const float2*)x2, (const float2*)y2, n, partials);
-  k_finish<<<1, 1024, 0, st>>>(partials, g, 6, weight, stage, S);
+                                              (const float2*)y1, (const float2*)x2, (const float2*)y2, n, red);
   return cudaGetLastError();
 }
 
 cudaError_t adj_hess_epi(int prec, const void* phi, const void* p, void* q, long long n, double eta, double lam,
-                         double weight, AdjScalars* S, double* partials, int max_blocks, cudaStream_t st) {
-  const int g = grid_of(n, max_blocks);
+                         double weight, const AdjWork& w, cudaStream_t st) {
+  const int g = grid_of(n, kAdjMaxBlocks);
+  const AdjRed red = {w.partials, w.ticket, weight, ADJ_PQ, w.S};
   if (prec == 1)
-    k_hess_epi<double2><<<g, kDotThreads, 0, st>>>((const double2*)phi, (const double2*)p, (double2*)q, n, eta, lam,
-                                                   partials);
+    k_hess_epi<double2><<<g, kDotThreads, 0, st>>>((const double2*)phi, (const double2*)p, (double2*)q, n, eta, lam, red);
   else
-    k_hess_epi<float2><<<g, kDotThreads, 0, st>>>((const float2*)phi, (const float2*)p, (float2*)q, n, eta, lam,
-                                                  partials);
-  k_finish<<<1, 1024, 0, st>>>(partials, g, 6, weight, ADJ_PQ, S);
+    k_hess_epi<float2><<<g, kDotThreads, 0, st>>>((const float2*)phi, (const float2*)p, (float2*)q, n, eta, lam, red);
   return cudaGetLastError();
 }
 
 cudaError_t adj_step(int prec, void* z, void* r, const void* p, const void* q, const void* phi, long long n,
-                     double weight, AdjScalars* S, double* partials, int max_blocks, cudaStream_t st) {
-  const int g = grid_of(n, max_blocks);
+                     double weight, const AdjWork& w, cudaStream_t st) {
+  const int g = grid_of(n, kAdjMaxBlocks);
+  const AdjRed red = {w.partials, w.ticket, weight, ADJ_RR, w.S};
   if (prec == 1)
     k_step<double2><<<g, kDotThreads, 0, st>>>((double2*)z, (double2*)r, (const double2*)p, (const double2*)q,
-                                               (const double2*)phi, n, S, partials);
+                                               (const double2*)phi, n, red);
   else
     k_step<float2><<<g, kDotThreads, 0, st>>>((float2*)z, (float2*)r, (const float2*)p, (const float2*)q,
-                                              (const float2*)phi, n, S, partials);
-  k_finish<<<1, 1024, 0, st>>>(partials, g, 2, weight, ADJ_RR, S);
+                                              (const float2*)phi, n, red);
   return cudaGetLastError();
 }
 

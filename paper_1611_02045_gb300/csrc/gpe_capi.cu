@@ -663,7 +663,6 @@ extern "C" gpe_status gpe_precond(gpe_ctx* c, const void* phi, const void* r, do
   return run_PC(c, b, r, alpha, out, c->ctl_api, false, c->st);
 }
 
-constexpr int kAdjMaxBlocks = 1024;
 constexpr int kAdjCheckEvery = 4;  // iterations between host reads of the scalars
 
 static gpe_status tangent_solve(gpe_ctx* c, const void* phi, const void* rhs, void* z, double tol, int max_iter,
@@ -673,10 +672,11 @@ static gpe_status tangent_solve(gpe_ctx* c, const void* phi, const void* rhs, vo
   if (!c->adj_s) {
     for (auto& a : c->adj) GPE_CU(c, cudaMalloc(&a, bytes));
     GPE_CU(c, cudaMalloc(&c->adj_s, sizeof(AdjScalars)));
-    GPE_CU(c, cudaMalloc(&c->adj_partials, sizeof(double) * 6 * kAdjMaxBlocks));
+    GPE_CU(c, cudaMalloc(&c->adj_partials, sizeof(double) * 8 * kAdjMaxBlocks));
   }
   void *r = c->adj[0], *y = c->adj[1], *p = c->adj[2], *q = c->adj[3];
   AdjScalars* S = c->adj_s;
+  const AdjWork aw = {S, c->adj_partials, c->ticket};
   const long long N = c->N;
   const double w = c->weight;
   cudaStream_t st = c->st;
@@ -695,15 +695,14 @@ static gpe_status tangent_solve(gpe_ctx* c, const void* phi, const void* rhs, vo
   GPE_CU(c, cudaMemsetAsync(z, 0, bytes, st));
   GPE_CU(c, cudaMemsetAsync(p, 0, bytes, st));
   // r = P rhs, bb = ||r||^2
-  GPE_CU(c, adj_dots(prec, phi, rhs, nullptr, nullptr, nullptr, nullptr, N, w, ADJ_PROJ, S, c->adj_partials,
-                     kAdjMaxBlocks, st));
+  GPE_CU(c, adj_dots(prec, phi, rhs, nullptr, nullptr, nullptr, nullptr, N, w, ADJ_PROJ, aw, st));
   GPE_CU(c, adj_proj(prec, rhs, r, phi, N, S, st));
-  GPE_CU(c, adj_dots(prec, r, r, nullptr, nullptr, nullptr, nullptr, N, w, ADJ_BB, S, c->adj_partials, kAdjMaxBlocks, st));
+  GPE_CU(c, adj_dots(prec, r, r, nullptr, nullptr, nullptr, nullptr, N, w, ADJ_BB, aw, st));
   IterBufs b = iter_bufs(c, prec);
   b.phi = const_cast<void*>(phi);
   // y = P_C r; p = P y
   if ((s = run_PC(c, b, r, alpha, y, c->ctl_api, false, st)) != GPE_OK) return s;
-  GPE_CU(c, adj_dots(prec, phi, y, r, y, r, phi, N, w, ADJ_RY_FIRST, S, c->adj_partials, kAdjMaxBlocks, st));
+  GPE_CU(c, adj_dots(prec, phi, y, r, y, r, phi, N, w, ADJ_RY_FIRST, aw, st));
   GPE_CU(c, adj_dir(prec, p, y, phi, N, S, st));
   AdjScalars hs = s0;
   int it = 0;
@@ -714,12 +713,12 @@ static gpe_status tangent_solve(gpe_ctx* c, const void* phi, const void* rhs, vo
       if (hs.stop || it >= max_iter) break;
     }
     // q = P K p;  a = Re<r, y> / Re<p, q>;  z += a p;  r -= a q
-    if ((s = run_H(c, prec, phi, p, q, c->ctl_api)) != GPE_OK) return s;
-    GPE_CU(c, adj_hess_epi(prec, phi, p, q, N, c->prob.eta, lam, w, S, c->adj_partials, kAdjMaxBlocks, st));
-    GPE_CU(c, adj_step(prec, z, r, p, q, phi, N, w, S, c->adj_partials, kAdjMaxBlocks, st));
+    if ((s = run_H(c, prec, phi, p, q, c->ctl_api, false)) != GPE_OK) return s;
+    GPE_CU(c, adj_hess_epi(prec, phi, p, q, N, c->prob.eta, lam, w, aw, st));
+    GPE_CU(c, adj_step(prec, z, r, p, q, phi, N, w, aw, st));
     // y = P_C r;  beta = Re<r, P y> / previous;  p = P y + beta p
     if ((s = run_PC(c, b, r, alpha, y, c->ctl_api, false, st)) != GPE_OK) return s;
-    GPE_CU(c, adj_dots(prec, phi, y, r, y, r, phi, N, w, ADJ_RY, S, c->adj_partials, kAdjMaxBlocks, st));
+    GPE_CU(c, adj_dots(prec, phi, y, r, y, r, phi, N, w, ADJ_RY, aw, st));
     GPE_CU(c, adj_dir(prec, p, y, phi, N, S, st));
     ++it;
   }

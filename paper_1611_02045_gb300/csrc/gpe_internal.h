@@ -226,13 +226,18 @@ struct AdjScalars {
   int iters;
 };
 enum AdjStage { ADJ_PROJ = 0, ADJ_BB = 1, ADJ_PQ = 2, ADJ_RR = 3, ADJ_RY = 4, ADJ_RY_FIRST = 5 };
+constexpr int kAdjMaxBlocks = 1024;
+struct AdjWork {
+  AdjScalars* S;
+  double* partials;  // [kAdjMaxBlocks][8]
+  unsigned* ticket;  // the context's reduction ticket (zero between kernels)
+};
 cudaError_t adj_dots(int prec, const void* x0, const void* y0, const void* x1, const void* y1, const void* x2,
-                     const void* y2, long long n, double weight, int stage, AdjScalars* S, double* partials,
-                     int max_blocks, cudaStream_t st);
+                     const void* y2, long long n, double weight, int stage, const AdjWork& w, cudaStream_t st);
 cudaError_t adj_hess_epi(int prec, const void* phi, const void* p, void* q, long long n, double eta, double lam,
-                         double weight, AdjScalars* S, double* partials, int max_blocks, cudaStream_t st);
+                         double weight, const AdjWork& w, cudaStream_t st);
 cudaError_t adj_step(int prec, void* z, void* r, const void* p, const void* q, const void* phi, long long n,
-                     double weight, AdjScalars* S, double* partials, int max_blocks, cudaStream_t st);
+                     double weight, const AdjWork& w, cudaStream_t st);
 cudaError_t adj_proj(int prec, const void* h_in, void* h_out, const void* phi, long long n, const AdjScalars* S,
                      cudaStream_t st);
 cudaError_t adj_dir(int prec, void* p, const void* y, const void* phi, long long n, const AdjScalars* S,
