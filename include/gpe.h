@@ -183,13 +183,14 @@ gpe_status gpe_apply_H(gpe_ctx* ctx, const void* phi_dev, const void* f_dev, voi
  * contexts with nx == ny in [32, 256] only.  Global memory is read and written
  * once per point (the output is written by the row part and completed by the
  * column part while still in L2).  Forms, by plan mode 3 of gpe_set_plan:
- *  - single precision, 256 x 256, f == phi, 16-byte aligned fields and V,
- *    E = 16 with width 16 (the default): a dataflow of row units and column
- *    units (16 lines each) taken by persistent blocks on every SM from one
- *    ticket queue, inputs copied by the TMA; a field's column units add their
- *    part after its row units have stored theirs.  Uses a counter array of the
- *    context (nbatch + 2 ints, allocated on first use and when the batch
- *    grows; zero between calls), so one such call runs at a time per context;
+ *  - single precision, n = 64, 128 or 256, 16-byte aligned f, out and V, at
+ *    least 2^21 (n = 256) or 3 2^20 points in the batch, E = 16 with width 16 (the
+ *    default): a dataflow of row units and column units (4096 points each)
+ *    taken by persistent blocks on every SM from one ticket queue, inputs
+ *    copied by the TMA; a field's column units add their part after its row
+ *    units have stored theirs.  Uses a counter array of the context (nbatch + 2
+ *    ints, reallocated when a batch outgrows it; not used under stream capture
+ *    then; zero between calls), so one such call runs at a time per context;
  *  - otherwise one thread-block cluster per field (16 rows per CTA) in
  *    distributed shared memory; in single precision with n >= 64 and 16-byte
  *    aligned phi and f the resident clusters loop over the fields and copy the

@@ -381,6 +381,13 @@ extern "C" gpe_status gpe_create(const gpe_problem* prob, const double* V, void*
       c->err = "cudaMalloc persistent workspace"; return fail(GPE_ERR_CUDA);
     }
   }
+  if (c->work == 0) {  // counters of the dataflow form, for up to 1022 planes without another allocation
+    c->hflow_cap = 1024;
+    if (cudaMalloc(&c->hflow_ctr, c->hflow_cap * sizeof(int)) != cudaSuccess ||
+        cudaMemset(c->hflow_ctr, 0, c->hflow_cap * sizeof(int)) != cudaSuccess) {
+      c->err = "cudaMalloc dataflow counters"; return fail(GPE_ERR_CUDA);
+    }
+  }
   cudaMemset(c->ctl_solve, 0, sizeof(Ctl));
   cudaMemset(c->ctl_api, 0, sizeof(Ctl));
   cudaMemset(c->ticket, 0, 4 * sizeof(unsigned));
@@ -402,16 +409,64 @@ extern "C" const char* gpe_last_error(const gpe_ctx* c) { return c ? c->err.c_st
 // accumulated; the last one writes `out` (or t) and finalises the energy terms.
 // moments = false: H phi as a plain operator (gpe_apply_H); the passes skip the
 // energy moments and the scalar step that only gpe_energy and the solver read.
+// The x and y parts of H phi on complex64 planes as a dataflow (gpe_hflow.cu):
+// nplanes planes of the context's nx x ny, V one plane (vstride 0) or one per plane.
+// The dataflow needs enough units to fill its pipeline (a unit is 4096 points, 304
+// blocks hold two each); below these sizes the other forms are faster:
+//  * 3D, against an x and a y pass: 2^22 points (256 x 256 x 64: 54 against 68 us,
+//    64 x 256 x 256: 66 / 72; with 2^21, 128^3: 39.5 / 37.1, 64 x 64 x 512: 46.6 / 41.1);
+//  * batches, against the streaming clusters: 2^21 points at 256^2 (32 fields: 27 / 31
+//    us; 16 fields: 22.6 / 20.6), 3 2^20 at 64^2 and 128^2 (1024 x 64^2: 38 / 46 us, 333 x
+//    128^2: 43 / 55; with fewer, 333 x 64^2: 25 / 20, 128 x 128^2: 28 / 26).
+static bool flow_pays(const gpe_ctx* c, long long points) {
+  if (c->dim == 3) return points >= (1ll << 22);
+  return points >= (c->n[0] == 256 ? 1ll << 21 : 3ll << 20);
+}
+static gpe_status try_flow(gpe_ctx* c, int nplanes, long long vstride, const void* phi, const void* f, void* out,
+                           bool* used) {
+  const PrecBufs& b = c->pb[0];
+  FlowHArgs a;
+  a.mx = c->n[0]; a.my = c->n[1]; a.nbatch = nplanes;
+  a.stride = (long long)c->n[0] * c->n[1]; a.vstride = vstride;
+  a.eta = c->prob.eta; a.omega = c->prob.omega;
+  a.xi = b.xi[0]; a.xiy = b.xi[1]; a.xc = b.xc[0]; a.yc = b.xc[1]; a.twx = b.tw[0]; a.twy = b.tw[1];
+  a.V = b.V; a.phi = phi; a.f = f; a.out = out;
+  // counters: allocated (zeroed) with the context, again when the batch grows; the kernel leaves them zero
+  const size_t need = h_batch_flow_counters(nplanes);
+  if ((size_t)c->hflow_cap < need) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    GPE_CU(c, cudaStreamIsCapturing(c->st, &cs));
+    if (cs != cudaStreamCaptureStatusNone) return GPE_OK;  // no allocation under capture: the other forms
+    const size_t cap = need > 2 * (size_t)c->hflow_cap ? need : 2 * (size_t)c->hflow_cap;
+    if (c->hflow_ctr) GPE_CU(c, cudaFree(c->hflow_ctr));
+    c->hflow_ctr = nullptr;
+    c->hflow_cap = 0;
+    GPE_CU(c, cudaMalloc(&c->hflow_ctr, cap * sizeof(int)));
+    GPE_CU(c, cudaMemsetAsync(c->hflow_ctr, 0, cap * sizeof(int), c->st));
+    c->hflow_cap = (int)cap;
+  }
+  a.ctr = c->hflow_ctr;
+  a.ctr_cap = c->hflow_cap;
+  a.status = &c->ctl_api->status;
+  GPE_CU(c, launch_h_batch_flow(a, c->st, used));
+  return GPE_OK;
+}
+
 static gpe_status run_H(gpe_ctx* c, int prec, const void* phi, const void* f, void* out, Ctl* ctl,
                         bool moments = true) {
+  bool flowed = false;
+  if (prec == 0 && !moments && c->dim == 3 && flow_pays(c, c->N)) {
+    const gpe_status s = try_flow(c, c->n[2], (long long)c->n[0] * c->n[1], phi, f, c->pb[0].t, &flowed);
+    if (s != GPE_OK) return s;
+  }
   PassArgs a = base_args(c, prec, 0, prec);
   a.ctl = ctl; a.phi = phi; a.f = f; a.t = c->pb[prec].t;
   a.nomoments = moments ? 0 : 1;
   // fields above 64 MB (beyond L2 with the operator's other arrays): the x pass
   // prefetches the rows of the block one wave ahead (two blocks per SM)
   if ((double)c->N * (prec == 0 ? 8.0 : 16.0) > 64.0 * 1024 * 1024) a.pf = 2 * c->nsm;
-  GPE_CU(c, launch(prec, P_HX, a, c->st));
-  for (int ax = 1; ax < c->dim; ++ax) {
+  if (!flowed) GPE_CU(c, launch(prec, P_HX, a, c->st));
+  for (int ax = flowed ? 2 : 1; ax < c->dim; ++ax) {
     PassArgs b = base_args(c, prec, ax, prec);
     b.ctl = ctl; b.phi = phi; b.f = f; b.t = c->pb[prec].t;
     b.nomoments = a.nomoments;
@@ -446,22 +501,10 @@ extern "C" gpe_status gpe_apply_H_batch(gpe_ctx* c, int nbatch, const void* phi,
   a.phi = phi; a.f = f; a.out = out;
   a.E = c->hbatch_E;
   a.rows = c->hbatch_rows;
-  if (prec == 0 && a.M == 256 && a.E == 16 && a.rows == 16 && phi == f) {
-    // the dataflow form's counters: allocated (zeroed) on first use and when the batch grows;
-    // the kernel leaves them zero
-    const size_t need = h_batch_flow_counters(nbatch);
-    if ((size_t)c->hflow_cap < need) {
-      const size_t cap = need > 2 * (size_t)c->hflow_cap ? need : 2 * (size_t)c->hflow_cap;
-      if (c->hflow_ctr) GPE_CU(c, cudaFree(c->hflow_ctr));
-      c->hflow_ctr = nullptr;
-      c->hflow_cap = 0;
-      GPE_CU(c, cudaMalloc(&c->hflow_ctr, cap * sizeof(int)));
-      GPE_CU(c, cudaMemsetAsync(c->hflow_ctr, 0, cap * sizeof(int), c->st));
-      c->hflow_cap = (int)cap;
-    }
-    a.flow_ctr = c->hflow_ctr;
-    a.flow_cap = c->hflow_cap;
-    a.status = &c->ctl_api->status;
+  if (prec == 0 && a.E == 16 && a.rows == 16 && flow_pays(c, nbatch * c->N)) {
+    bool used = false;
+    const gpe_status s = try_flow(c, nbatch, 0, phi, f, out, &used);
+    if (s != GPE_OK || used) return s;
   }
   GPE_CU(c, launch_cluster_apply_H(prec, a, c->st));
   return GPE_OK;

@@ -194,6 +194,25 @@ cudaError_t launch_group_split_e4(Pass pass, const PassArgs& a, cudaStream_t st)
 struct ClusterHArgs;
 cudaError_t launch_cluster_apply_H(int is_double, const ClusterHArgs& a, cudaStream_t st);
 
+// H phi on complex64 planes (the fields of a 2D batch, or the x and y parts on the z
+// planes of a 3D field) as a dataflow of row and column units (gpe_hflow.cu); *used =
+// false when the call does not qualify: sides 64, 128 or 256, f, out and V 16-byte
+// aligned.  out must not overlap phi or f.
+struct FlowHArgs {
+  int mx, my, nbatch;
+  long long stride;   // elements between consecutive planes
+  long long vstride;  // elements between the planes of V (0: one V for all)
+  double eta, omega;
+  const void *xi, *xiy, *xc, *yc, *twx, *twy;  // float tables of both axes
+  const void *V, *phi, *f;
+  void* out;
+  int* ctr;     // zeroed counters, at least h_batch_flow_counters(nbatch) ints
+  int ctr_cap;
+  int* status;  // device int set to GPE_ERR_TIMEOUT when a bounded wait gives up (or null)
+};
+cudaError_t launch_h_batch_flow(const FlowHArgs& a, cudaStream_t st, bool* used);
+size_t h_batch_flow_counters(int nbatch);
+
 // The complex64 phase of a 2D solve in one thread-block cluster's shared
 // memory (gpe_csolve.cuh; M = nx = ny in [32, 256]).
 struct ClusterSolveArgs;
