@@ -114,25 +114,29 @@ __device__ __forceinline__ void cs_yunit(const cgc::cluster_group& cl, int rank,
 template <int ROLE>
 __device__ __forceinline__ void cs_reduce(const cgc::cluster_group& cl, int rank, int csize, const Acc* acc,
                                           Acc* part, int& parity, Acc* red_sm, double weight, double* tot) {
-  constexpr int K = Moments<ROLE>::K;
+  constexpr int K = Moments<ROLE>::K, lg = Slots<K>::lg, P = Slots<K>::P;
   constexpr unsigned MAXMASK = Moments<ROLE>::MAX;
   Acc v[K];
 #pragma unroll
   for (int k = 0; k < K; ++k) v[k] = acc[k];
-  block_reduce<K, MAXMASK, false>(v, red_sm + parity * 32 * kMaxMoments);
   Acc* p0 = cl.map_shared_rank(part, 0u) + (size_t)parity * kCSRows * kMaxMoments;
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) p0[rank * kMaxMoments + k] = v[k];
-  }
+  block_reduce<K, MAXMASK, false>(v, red_sm + parity * kRedSlots, [&](int k, Acc t) { p0[rank * kMaxMoments + k] = t; });
   cl.sync();
   if (threadIdx.x < 32) {
-    // lane r takes CTA r's partials; fixed-order shuffle tree across the lanes
-    const int lane = threadIdx.x;
+    // lane l takes slot l mod P of the CTAs l / P, l / P + 32 / P, ...
+    const int lane = threadIdx.x, k = lane & (P - 1);
+    constexpr int U = kCSRows * P / 32 > 0 ? kCSRows * P / 32 : 1;
+    Acc x[U], t{0.0f, 0.0f};
 #pragma unroll
-    for (int k = 0; k < K; ++k) v[k] = lane < csize ? p0[lane * kMaxMoments + k] : Acc{0.0f, 0.0f};
-    warp_tree<K, MAXMASK>(v);
-    totals<K, Moments<ROLE>::W>(v, weight, tot);
+    for (int i = 0; i < U; ++i) {
+      const int c = (lane >> lg) + i * (32 >> lg);
+      x[i] = (c < csize && k < K) ? p0[c * kMaxMoments + k] : Acc{0.0f, 0.0f};
+    }
+#pragma unroll
+    for (int i = 0; i < U; ++i) t = red_op<MAXMASK>(t, x[i], k);
+#pragma unroll
+    for (int o = P; o < 32; o <<= 1) t = red_op<MAXMASK>(t, shfl_acc(0xffffffffu, t, o), k);
+    if (lane < K) tot[lane] = total<Moments<ROLE>::W>(t, weight, lane);
     __syncwarp();
   }
   parity ^= 1;
@@ -153,7 +157,7 @@ __global__ void __launch_bounds__((M / 8) * kCSRows) cluster_solve(ClusterSolveA
   float2* xs = r_s + R * M;  // exchange scratch, R * LS elements
   __shared__ Ctl S;
   __shared__ Acc part[2 * kCSRows * kMaxMoments];
-  __shared__ Acc red_sm[2 * 32 * kMaxMoments];  // two buffers, alternating with the reductions
+  __shared__ Acc red_sm[2 * kRedSlots];  // two buffers, alternating with the reductions
   __shared__ double tot[2][kMaxMoments];  // x and y totals of the operator under way
 
   const int row0 = rank * R;
@@ -199,7 +203,7 @@ __global__ void __launch_bounds__((M / 8) * kCSRows) cluster_solve(ClusterSolveA
     // ---- H phi_n (x pass folds in the retraction to phi_n) ----
     Scal sc = scal_of(&S, ax);
     zero();
-    xunit<float, float, float, M, P_HX>(ax, sc, 0, xsb, acc);
+    xunit<float, float, float, M, P_HX, 8, true>(ax, sc, 0, xsb, acc);
     cs_reduce<P_HX>(cl, rank, csize, acc, part, parity, red_sm, w, tot[0]);
     zero();
     cs_yunit<M, P_HMID>(cl, rank, phi_s, t_s, xs, ax, sc, acc);
@@ -209,22 +213,24 @@ __global__ void __launch_bounds__((M / 8) * kCSRows) cluster_solve(ClusterSolveA
     // ---- residual, stopping rule, P_C r_n ----
     sc = scal_of(&S, ax);
     zero();
-    xunit<float, float, float, M, P_C1>(ax, sc, 0, xsb, acc);
+    xunit<float, float, float, M, P_C1, 8, true>(ax, sc, 0, xsb, acc);
     cs_reduce<P_C1>(cl, rank, csize, acc, part, parity, red_sm, w, tot[0]);
     if (threadIdx.x < 32) finalize_C1(&S, tot[0], writer);
     __syncthreads();
     if (S.done) break;
+    sc = scal_of(&S, ax);  // taken afresh where they are used: registers are short across a pass
     cs_yunit<M, P_CCORE>(cl, rank, s_s, nullptr, xs, ax, sc, acc);
     cl.sync();
+    sc = scal_of(&S, ax);
     zero();
-    xunit<float, float, float, M, P_C3>(ax, sc, 0, xsb, acc);
+    xunit<float, float, float, M, P_C3, 8, true>(ax, sc, 0, xsb, acc);
     cs_reduce<P_C3>(cl, rank, csize, acc, part, parity, red_sm, w, tot[0]);
     if (threadIdx.x < 32) finalize_C3(&S, tot[0], writer);
     __syncthreads();
     // ---- p_n and the step size ----
     sc = scal_of(&S, ax);
     zero();
-    xunit<float, float, float, M, P_AX>(ax, sc, 0, xsb, acc);
+    xunit<float, float, float, M, P_AX, 8, true>(ax, sc, 0, xsb, acc);
     cs_reduce<P_AX>(cl, rank, csize, acc, part, parity, red_sm, w, tot[0]);
     zero();
     cs_yunit<M, P_AMID>(cl, rank, p_s, nullptr, xs, ax, sc, acc);

@@ -374,10 +374,17 @@ __global__ void __launch_bounds__(kNormThreads) k_init_norm(const C* __restrict_
     s_last = (atomicAdd(ticket, 1u) == gridDim.x - 1) ? 1 : 0;
   }
   __syncthreads();
-  if (!s_last || threadIdx.x != 0) return;
+  if (!s_last) return;
   __threadfence();
+  // FP64 additions are 64 cycles apart in one thread: the block shares them
+  acc = 0.0;
+  for (unsigned b = threadIdx.x; b < gridDim.x; b += blockDim.x) acc += __ldcg(partials + b);
+  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) sm[threadIdx.x >> 5] = acc;  // read by thread 0 before s_last's barrier
+  __syncthreads();
+  if (threadIdx.x != 0) return;
   double tot = 0.0;
-  for (unsigned b = 0; b < gridDim.x; ++b) tot += __ldcg(partials + b);
+  for (int w = 0; w < kNormThreads / 32; ++w) tot += sm[w];
   ctl->cc = num(1.0 / sqrt(weight * tot));
   ctl->ss = num(0.0);
   ctl->retract = 1;

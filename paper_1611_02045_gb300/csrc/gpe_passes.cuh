@@ -80,9 +80,12 @@ __device__ __forceinline__ Acc acc_max(Acc a, Acc b) {
   return (b.hi > a.hi || (b.hi == a.hi && b.lo > a.lo)) ? b : a;
 }
 
+// Slot k's reduction (k may differ between lanes).
 template <unsigned MAXMASK>
 __device__ __forceinline__ Acc red_op(Acc a, Acc b, int k) {
-  return ((MAXMASK >> k) & 1u) ? acc_max(a, b) : acc_add(a, b);
+  const Acc s = acc_add(a, b);
+  if constexpr (MAXMASK == 0u) return s;
+  return ((MAXMASK >> k) & 1u) ? acc_max(a, b) : s;
 }
 
 // Two double-single additions at once on the packed two-wide FP32 pipe: lane by
@@ -113,69 +116,104 @@ __device__ __forceinline__ void acc_add2(Acc& a0, Acc& a1, Acc b0, Acc b1) {
   a1 = Acc{H.y, Lo.y};
 }
 
-// v[k] = red_op(v[k], w[k]) for every slot; pairs of sum slots go through acc_add2.
-template <int K, unsigned MAXMASK>
-__device__ __forceinline__ void red_all(Acc (&v)[K], const Acc (&w)[K]) {
-#pragma unroll
-  for (int k = 0; k < K; k += 2) {
-    if (k + 1 < K && !((MAXMASK >> k) & 1u) && !((MAXMASK >> (k + 1)) & 1u)) {
-      acc_add2(v[k], v[k + 1], w[k], w[k + 1]);
-    } else {
-      v[k] = red_op<MAXMASK>(v[k], w[k], k);
-      if (k + 1 < K) v[k + 1] = red_op<MAXMASK>(v[k + 1], w[k + 1], k + 1);
-    }
-  }
-}
-
 __device__ __forceinline__ Acc shfl_acc(unsigned mask, Acc v, int o) {
   return Acc{__shfl_xor_sync(mask, v.hi, o), __shfl_xor_sync(mask, v.lo, o)};
 }
 
-// Fixed-order butterfly over the 32 lanes of a warp (lanes beyond the data
-// hold the identity, 0, which also serves the max slots: they are >= 0).
+// Slots padded to a power of two.
+template <int K> struct Slots {
+  static constexpr int lg = K <= 1 ? 0 : K <= 2 ? 1 : K <= 4 ? 2 : K <= 8 ? 3 : 4;
+  static constexpr int P = 1 << lg;
+};
+
+// The K slots reduced over a full warp in a fixed order: lane l returns the total
+// of slot l >> (5 - lg).  Each of the first lg steps halves the slots a lane keeps
+// along with the lanes, so K = 9 takes 16 additions, not 45.  These sums are short
+// on purpose: in the last block of a pass, and in every pass of a resident solve,
+// they run once through, and their time is that of fetching the instructions (a
+// fully unrolled tree over all slots, in several copies, was most of the code:
+// cluster solve 39 -> 26 us per iteration at 64^2, 60 -> 48 at 256^2; graph loop
+// 487 -> 458 us per refinement iteration at 128^3, 85 -> 75 at 256^2).
 template <int K, unsigned MAXMASK>
-__device__ __forceinline__ void warp_tree(Acc (&v)[K]) {
+__device__ __forceinline__ Acc warp_slots(const Acc (&v)[K]) {
+  constexpr int lg = Slots<K>::lg, P = Slots<K>::P;
+  const int lane = threadIdx.x & 31;
+  Acc w[P];
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    Acc w[K];
+  for (int k = 0; k < P; ++k) w[k] = (k < K && !((MAXMASK >> k) & 1u)) ? v[k < K ? k : 0] : Acc{0.0f, 0.0f};
 #pragma unroll
-    for (int k = 0; k < K; ++k) w[k] = shfl_acc(0xffffffffu, v[k], o);
-    red_all<K, MAXMASK>(v, w);
+  for (int st = 0; st < lg; ++st) {
+    const int o = 16 >> st, h = P >> (st + 1);
+    const bool up = lane & o;
+#pragma unroll
+    for (int j = 0; j < h; j += 2) {
+      const Acc k0 = up ? w[j + h] : w[j], s0 = up ? w[j] : w[j + h];
+      const Acc r0 = shfl_acc(0xffffffffu, s0, o);
+      if (j + 1 < h) {
+        const Acc k1 = up ? w[j + 1 + h] : w[j + 1], s1 = up ? w[j + 1] : w[j + 1 + h];
+        const Acc r1 = shfl_acc(0xffffffffu, s1, o);
+        w[j] = k0;
+        w[j + 1] = k1;
+        acc_add2(w[j], w[j + 1], r0, r1);
+      } else {
+        w[j] = acc_add(k0, r0);
+      }
+    }
   }
+#pragma unroll
+  for (int o = 16 >> lg; o > 0; o >>= 1) w[0] = acc_add(w[0], shfl_acc(0xffffffffu, w[0], o));
+  if constexpr (MAXMASK != 0u) {
+#pragma unroll
+    for (int k = 0; k < K; ++k)
+      if ((MAXMASK >> k) & 1u) {
+        Acc x = v[k];
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) x = acc_max(x, shfl_acc(0xffffffffu, x, o));
+        if ((lane >> (5 - lg)) == k) w[0] = x;
+      }
+  }
+  return w[0];
 }
 
-// Block total of v[k] (fixed tree); valid in thread 0 on return.  Warp sums
-// by shuffles, then warp 0 combines the per-warp sums with a second shuffle
-// tree (no serial loop over warps).
+// Block totals: sink(k, total of slot k) is called once per slot by a thread of
+// warp 0 (thread k where the block has a full warp).  red_sm: kRedSlots elements.
 // LEAD = false skips the barrier that protects red_sm from the previous call's
 // readers: for callers that alternate between two red_sm buffers, whose other
 // barriers already order a buffer's readers before its next writers.
-template <int K, unsigned MAXMASK, bool LEAD = true>
-__device__ __forceinline__ void block_reduce(Acc (&v)[K], Acc* red_sm) {
+constexpr int kRedSlots = 256;
+template <int K, unsigned MAXMASK, bool LEAD = true, typename Sink>
+__device__ __forceinline__ void block_reduce(const Acc (&v)[K], Acc* red_sm, Sink sink) {
+  constexpr int lg = Slots<K>::lg, P = Slots<K>::P;
   // blockDim.x is a power of two: either a multiple of 32 or one partial warp
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-  const int width = blockDim.x < 32 ? (int)blockDim.x : 32;
-  const unsigned mask = width == 32 ? 0xffffffffu : ((1u << width) - 1u);
+  if (blockDim.x >= 32) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    Acc t = warp_slots<K, MAXMASK>(v);
+    if (nw == 1) {
+      const int src = (lane & (P - 1)) << (5 - lg);
+      t = Acc{__shfl_sync(0xffffffffu, t.hi, src), __shfl_sync(0xffffffffu, t.lo, src)};
+    } else {
+      if constexpr (LEAD) __syncthreads();
+      if ((lane & ((32 >> lg) - 1)) == 0) red_sm[warp * P + (lane >> (5 - lg))] = t;
+      __syncthreads();
+      if (warp != 0) return;
+      const int k = lane & (P - 1);
+      t = Acc{0.0f, 0.0f};  // also the identity of the maxima, which are >= 0
+#pragma unroll 2
+      for (int w = lane >> lg; w < nw; w += 32 >> lg) t = red_op<MAXMASK>(t, red_sm[w * P + k], k);
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    if (o < width) {
-      Acc w[K];
-#pragma unroll
-      for (int k = 0; k < K; ++k) w[k] = shfl_acc(mask, v[k], o);
-      red_all<K, MAXMASK>(v, w);
+      for (int o = P; o < 32; o <<= 1) t = red_op<MAXMASK>(t, shfl_acc(0xffffffffu, t, o), k);
     }
-  }
-  if (nw == 1) return;
-  if constexpr (LEAD) __syncthreads();
-  if (lane == 0) {
+    if (lane < K) sink(lane, t);
+  } else {
+    if constexpr (LEAD) __syncthreads();
 #pragma unroll
-    for (int k = 0; k < K; ++k) red_sm[warp * K + k] = v[k];
-  }
-  __syncthreads();
-  if (warp == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) v[k] = lane < nw ? red_sm[lane * K + k] : Acc{0.0f, 0.0f};
-    warp_tree<K, MAXMASK>(v);
+    for (int k = 0; k < K; ++k) red_sm[threadIdx.x * K + k] = v[k];
+    __syncthreads();
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
+      Acc t = red_sm[k];
+      for (int j = 1; j < (int)blockDim.x; ++j) t = red_op<MAXMASK>(t, red_sm[j * K + k], k);
+      sink(k, t);
+    }
   }
 }
 
@@ -192,40 +230,63 @@ template <> struct Moments<P_C3> { static constexpr int K = 6; static constexpr 
 template <> struct Moments<P_AX> { static constexpr int K = 9; static constexpr unsigned MAX = 0u, W = 511u; };
 template <> struct Moments<P_AMID> { static constexpr int K = 1; static constexpr unsigned MAX = 0u, W = 1u; };
 
-// Totals in FP64, times the weight where W says so, into out[] (shared memory).
-// v holds the block's totals in every lane of warp 0 (block_reduce); each lane
-// converts one slot: an FP64 instruction occupies its sub-partition's pipe for
-// 64 cycles whatever the number of active lanes, so one thread converting K
-// slots in turn would take K times as long.
-template <int K, unsigned W>
-__device__ __forceinline__ void totals(const Acc (&v)[K], double weight, double* out) {
-  const int lane = threadIdx.x, width = blockDim.x < 32 ? (int)blockDim.x : 32;
-  if (lane >= 32) return;
-  for (int b = 0; b < K; b += width) {
-    Acc x = v[0];
-#pragma unroll
-    for (int k = 1; k < K; ++k)
-      if (b + lane == k) x = v[k];
-    if (b + lane < K) out[b + lane] = acc_to_double(x) * (((W >> (b + lane)) & 1u) ? weight : 1.0);
-  }
+// A total in FP64, times the weight where W says so.  Each thread converts its own
+// slot: an FP64 instruction occupies its sub-partition's pipe for 64 cycles
+// whatever the number of active lanes, so one thread converting K slots in turn
+// would take K times as long.
+template <unsigned W>
+__device__ __forceinline__ double total(Acc x, double weight, int k) {
+  return acc_to_double(x) * (((W >> k) & 1u) ? weight : 1.0);
 }
 
-// Sum of a region's block partials in a fixed order (this thread's share).
-// L2-coherent loads, unrolled so that several blocks' partials are in flight
-// at once.
-template <int K, unsigned MAXMASK>
-__device__ __forceinline__ void sum_partials(const Acc* part, int nb, Acc (&w)[K]) {
-#pragma unroll
-  for (int k = 0; k < K; ++k) w[k] = Acc{0.0f, 0.0f};
-#pragma unroll 4
-  for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-    const float2* pb = reinterpret_cast<const float2*>(part + (size_t)b * kMaxMoments);
-#pragma unroll
-    for (int k = 0; k < K; ++k) {
-      const float2 x = __ldcg(pb + k);
-      w[k] = red_op<MAXMASK>(w[k], Acc{x.x, x.y}, k);
+// Sums of block partials in a fixed order, K slots at once: slot k adds elements
+// src(k)[b * kMaxMoments], b < nb(k); sink as for block_reduce.  A thread sums one
+// slot over a subset of the blocks, 16 L2-coherent loads in flight: a few hundred
+// instructions where one thread per block and all slots in registers takes
+// thousands.
+template <int K, unsigned MAXMASK, typename Src, typename Nb, typename Sink>
+__device__ __forceinline__ void sum_partials(Src src, Nb nb, Acc* red_sm, Sink sink) {
+  constexpr int lg = Slots<K>::lg, P = Slots<K>::P, U = 16;
+  if (blockDim.x < 32) {
+    for (int k = threadIdx.x; k < K; k += blockDim.x) {
+      const float2* p = reinterpret_cast<const float2*>(src(k));
+      Acc t{0.0f, 0.0f};
+      for (int b = 0; b < nb(k); ++b) {
+        const float2 x = __ldcg(p + (size_t)b * kMaxMoments);
+        t = red_op<MAXMASK>(t, Acc{x.x, x.y}, k);
+      }
+      sink(k, t);
     }
+    return;
   }
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int k = lane & (P - 1), J = (int)blockDim.x >> lg;
+  const int n = k < K ? nb(k) : 0;
+  const float2* p = reinterpret_cast<const float2*>(src(k < K ? k : 0));
+  Acc t{0.0f, 0.0f};
+  for (int b0 = threadIdx.x >> lg; b0 < n; b0 += U * J) {
+    float2 x[U];
+#pragma unroll
+    for (int i = 0; i < U; ++i)
+      x[i] = b0 + i * J < n ? __ldcg(p + (size_t)(b0 + i * J) * kMaxMoments) : make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int i = 0; i < U; ++i) t = red_op<MAXMASK>(t, Acc{x[i].x, x[i].y}, k);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int o = P; o < 32; o <<= 1) t = red_op<MAXMASK>(t, shfl_acc(0xffffffffu, t, o), k);
+  if (nw > 1) {
+    __syncthreads();  // earlier readers of red_sm
+    if (lane < P) red_sm[warp * P + lane] = t;
+    __syncthreads();
+    if (warp != 0) return;
+    t = Acc{0.0f, 0.0f};
+#pragma unroll 2
+    for (int w = lane >> lg; w < nw; w += 32 >> lg) t = red_op<MAXMASK>(t, red_sm[w * P + k], k);
+#pragma unroll
+    for (int o = P; o < 32; o <<= 1) t = red_op<MAXMASK>(t, shfl_acc(0xffffffffu, t, o), k);
+  }
+  if (lane < K) sink(lane, t);
 }
 
 // ---------------------------------------------------------------------------
@@ -422,7 +483,7 @@ __device__ __forceinline__ double delta_E(const StepPoly& P, double s, double c)
 // Newton's method on d/dt of the step polynomial delta_E (closed-form first
 // and second derivatives) from the model step t0; t0 is kept when the
 // curvature is not positive or the iterate leaves (0, pi/2].
-static __device__ double exact_step(double t0, const StepPoly& P) {
+static __device__ __noinline__ double exact_step(double t0, const StepPoly& P) {
   const double R = P.R, A = P.A, B = P.B, C = P.C, D = P.D;
   double t = t0;
   for (int it = 0; it < 30; ++it) {
@@ -594,7 +655,9 @@ __device__ __forceinline__ cplx<To> cconv(From v) { return cmk<cplx<To>>((To)v.x
 // One unit of a contiguous pass: lines unit*lpb .. unit*lpb + lpb - 1 (the
 // block has lpb * M/8 threads).  Adds this thread's reduction terms to acc[]
 // (Moments<ROLE>: sums, or maxima for the slots flagged in MAX).
-template <typename TF, typename TS, typename TD, int M, int ROLE, int EV = 8>
+// RES: a resident solve (fields in shared memory): operands are taken as they are
+// used, since nothing is gained by having them in flight early.
+template <typename TF, typename TS, typename TD, int M, int ROLE, int EV = 8, bool RES = false>
 __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long long unit, unsigned char* smraw,
                                       Acc* acc) {
   using CF = cplx<TF>;
@@ -642,15 +705,32 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
     const CD* __restrict__ p = static_cast<const CD*>(a.p);
     CS* __restrict__ phi_out = static_cast<CS*>(a.phi_out);
     CD pq[E];
+    if constexpr (RES) {
+      const TS cc = num_as<TS>(S.cc), ss = num_as<TS>(S.ss);
 #pragma unroll
-    for (int q = 0; q < E; ++q) {
-      const long long g = base + t + q * Tl;
-      ph[q] = phi[g];
-      vv[q] = V[g];
-      if (a.solver) pq[q] = p[g];
-      else v[q] = cconv<TF>(a.f ? f[g] : ph[q]);
+      for (int q = 0; q < E; ++q) {
+        const long long g = base + t + q * Tl;
+        CS x = phi[g];
+        if (retract) {
+          const CS d = cconv<TS>(p[g]);
+          x = cmk<CS>(cc * x.x + ss * d.x, cc * x.y + ss * d.y);
+          phi_out[g] = x;
+        }
+        ph[q] = x;
+        vv[q] = V[g];
+        v[q] = cconv<TF>(x);
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < E; ++q) {
+        const long long g = base + t + q * Tl;
+        ph[q] = phi[g];
+        vv[q] = V[g];
+        if (a.solver) pq[q] = p[g];
+        else v[q] = cconv<TF>(a.f ? f[g] : ph[q]);
+      }
     }
-    if (a.solver) {
+    if (!RES && a.solver) {
       if (S.done) return;
       const TS cc = num_as<TS>(S.cc), ss = num_as<TS>(S.ss);
 #pragma unroll
@@ -950,14 +1030,28 @@ __device__ __forceinline__ void sunit(const PassArgs& a, const Scal& S, long lon
 // us (256^2, complex64), 121 to 113 us (256^2, refinement) and 585 to 531 us
 // (128^3, refinement).
 // ---------------------------------------------------------------------------
+// All the sums of ROLE's operator, in the order its scalar step reads them: those of
+// the x pass, then of each further axis (KM per axis).
+template <int ROLE> struct OpSums { static constexpr int KX = Moments<ROLE>::K, KM = 0; };
+template <> struct OpSums<P_HMID> { static constexpr int KX = Moments<P_HX>::K, KM = Moments<P_HMID>::K; };
+template <> struct OpSums<P_AMID> { static constexpr int KX = Moments<P_AX>::K, KM = Moments<P_AMID>::K; };
+template <int ROLE> struct OpMasks {
+  static constexpr int KX = OpSums<ROLE>::KX, KM = OpSums<ROLE>::KM, K = KX + 2 * KM;
+  static constexpr unsigned WX = ROLE == P_HMID ? Moments<P_HX>::W : ROLE == P_AMID ? Moments<P_AX>::W : Moments<ROLE>::W;
+  static constexpr unsigned MAX =
+      ROLE == P_HMID ? Moments<P_HX>::MAX : ROLE == P_AMID ? Moments<P_AX>::MAX : Moments<ROLE>::MAX;
+  static constexpr unsigned W = WX | (((1u << (2 * KM)) - 1u) << KX);
+};
+
 // The scalar step of ROLE's operator, by warp 0 of the last block.
 template <int ROLE>
-__device__ __forceinline__ void run_scalar_step(const PassArgs& a, Ctl* c, const double (&tot)[3][kMaxMoments]) {
+__device__ __forceinline__ void run_scalar_step(const PassArgs& a, Ctl* c, const double* tot) {
   const Fin F = fin_of(a);
-  if constexpr (ROLE == P_HMID) finalize_H(c, F, tot[0], tot[1], tot[2], true);
-  else if constexpr (ROLE == P_C1) finalize_C1(c, tot[0], true);
-  else if constexpr (ROLE == P_C3) finalize_C3(c, tot[0], true);
-  else if constexpr (ROLE == P_AMID) finalize_A(c, F, tot[0], tot[1][0], tot[2][0], true);
+  constexpr int KX = OpSums<ROLE>::KX, KM = OpSums<ROLE>::KM;
+  if constexpr (ROLE == P_HMID) finalize_H(c, F, tot, tot + KX, tot + KX + KM, true);
+  else if constexpr (ROLE == P_C1) finalize_C1(c, tot, true);
+  else if constexpr (ROLE == P_C3) finalize_C3(c, tot, true);
+  else if constexpr (ROLE == P_AMID) finalize_A(c, F, tot, tot[KX], tot[KX + KM], true);
 }
 
 template <int ROLE>
@@ -966,58 +1060,48 @@ __device__ __forceinline__ void reduce_and_finish(const PassArgs& a, const Acc* 
   if (a.nomoments) return;  // uniform over the launch
   if constexpr (K > 0) {
     constexpr bool xpart = ROLE == P_HX || ROLE == P_AX, mid = ROLE == P_HMID || ROLE == P_AMID;
-    constexpr int KX = ROLE == P_AMID ? Moments<P_AX>::K : Moments<P_HX>::K;  // x totals a mid pass sums too
-    constexpr unsigned MX = ROLE == P_AMID ? Moments<P_AX>::MAX : Moments<P_HX>::MAX;
-    constexpr unsigned WX = ROLE == P_AMID ? Moments<P_AX>::W : Moments<P_HX>::W;
     // the P_C passes reduce only inside a solve
     if ((ROLE == P_C1 || ROLE == P_C3) && !a.solver) return;
-    __shared__ Acc red_sm[32 * (mid ? (K > KX ? K : KX) : K)];
-    __shared__ int s_last;
+    __shared__ Acc red_sm[kRedSlots];
     Acc v[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) v[k] = acc[k];
-    block_reduce<K, Moments<ROLE>::MAX>(v, red_sm);
     const int reg = (xpart || mid) ? a.axis : 0;
     Acc* part = acc_slots(a.partials);
-    if (threadIdx.x == 0) {
-#pragma unroll
-      for (int k = 0; k < K; ++k) part[reg * a.region + (size_t)blockIdx.x * kMaxMoments + k] = v[k];
-      if ((xpart || mid) && blockIdx.x == 0) a.nparts[reg] = (int)gridDim.x;
-    }
+    Acc* mine = part + reg * a.region + (size_t)blockIdx.x * kMaxMoments;
+    block_reduce<K, Moments<ROLE>::MAX>(v, red_sm, [&](int k, Acc t) { mine[k] = t; });
+    if ((xpart || mid) && blockIdx.x == 0 && threadIdx.x == 0) a.nparts[reg] = (int)gridDim.x;
     if (xpart || (mid && !a.last_axis)) return;
     if constexpr (!xpart) {
-      __shared__ double tot[3][kMaxMoments];
+      using OM = OpMasks<ROLE>;
+      __shared__ double tot[OM::K];
+      __shared__ int s_last;
       __shared__ Ctl sctl;
-      if (threadIdx.x == 0) {
+      if (threadIdx.x < 32) {  // the warp that stored the partials
         __threadfence();
-        const unsigned prev = atomicAdd(a.ticket, 1u);
-        s_last = (prev == gridDim.x - 1) ? 1 : 0;
+        if (full_warp()) __syncwarp();
+        else __syncwarp((1u << blockDim.x) - 1u);
+        if (threadIdx.x == 0) s_last = (atomicAdd(a.ticket, 1u) == gridDim.x - 1) ? 1 : 0;
       }
       __syncthreads();
       if (!s_last) return;
       __threadfence();
       constexpr int words = sizeof(Ctl) / 8;
       static_assert(sizeof(Ctl) % 8 == 0, "the control block is copied in 8-byte words");
-      const unsigned long long* src = reinterpret_cast<const unsigned long long*>(a.ctl);
+      const unsigned long long* from = reinterpret_cast<const unsigned long long*>(a.ctl);
       unsigned long long* cp = reinterpret_cast<unsigned long long*>(&sctl);
-      for (int i = threadIdx.x; i < words; i += blockDim.x) cp[i] = __ldcg(src + i);
-      if constexpr (mid) {
-        Acc w0[KX];
-        sum_partials<KX, MX>(part, __ldcg(a.nparts), w0);
-        for (int ax = 1; ax < a.dim; ++ax) {
-          Acc w1[K];
-          sum_partials<K, 0u>(part + ax * a.region, ax == a.axis ? (int)gridDim.x : __ldcg(a.nparts + ax), w1);
-          block_reduce<K, 0u>(w1, red_sm);
-          totals<K, Moments<ROLE>::W>(w1, a.weight, tot[ax]);
-        }
-        block_reduce<KX, MX>(w0, red_sm);
-        totals<KX, WX>(w0, a.weight, tot[0]);
-      } else {
-        Acc w[K];
-        sum_partials<K, Moments<ROLE>::MAX>(part, (int)gridDim.x, w);
-        block_reduce<K, Moments<ROLE>::MAX>(w, red_sm);
-        totals<K, Moments<ROLE>::W>(w, a.weight, tot[0]);
-      }
+      for (int i = threadIdx.x; i < words; i += blockDim.x) cp[i] = __ldcg(from + i);
+      auto region_of = [&](int k) { return k < OM::KX ? 0 : (k < OM::KX + OM::KM ? 1 : 2); };
+      auto src = [&](int k) {
+        const int r = region_of(k);
+        return part + r * a.region + (r == 0 ? k : (k - OM::KX) % (OM::KM ? OM::KM : 1));
+      };
+      auto nb = [&](int k) {
+        const int r = region_of(k);
+        if (mid && r != a.axis) return r < a.dim ? __ldcg(a.nparts + r) : 0;
+        return (int)gridDim.x;
+      };
+      sum_partials<OM::K, OM::MAX>(src, nb, red_sm, [&](int k, Acc t) { tot[k] = total<OM::W>(t, a.weight, k); });
       __syncthreads();  // totals and the control block copy
       if (threadIdx.x < (full_warp() ? 32 : 1)) {
         run_scalar_step<ROLE>(a, &sctl, tot);
@@ -1027,8 +1111,8 @@ __device__ __forceinline__ void reduce_and_finish(const PassArgs& a, const Acc* 
         }
       }
       __syncthreads();
-      unsigned long long* dst = reinterpret_cast<unsigned long long*>(a.ctl);
-      for (int i = threadIdx.x; i < words; i += blockDim.x) dst[i] = cp[i];
+      unsigned long long* to = reinterpret_cast<unsigned long long*>(a.ctl);
+      for (int i = threadIdx.x; i < words; i += blockDim.x) to[i] = cp[i];
     }
   }
 }

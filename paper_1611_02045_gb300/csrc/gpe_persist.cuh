@@ -69,21 +69,18 @@ template <int ROLE>
 __device__ __forceinline__ bool all_reduce(const PersistArgs& P, const Acc* acc, int& parity, double* tot) {
   constexpr int K = Moments<ROLE>::K;
   constexpr unsigned MAXMASK = Moments<ROLE>::MAX;
-  __shared__ Acc red_sm[32 * kMaxMoments];
+  __shared__ Acc red_sm[kRedSlots];
   Acc v[K];
 #pragma unroll
   for (int k = 0; k < K; ++k) v[k] = acc[k];
-  block_reduce<K, MAXMASK>(v, red_sm);
   Acc* part = acc_slots(P.partials) + (size_t)parity * gridDim.x * kMaxMoments;
-  if (threadIdx.x == 0) {
-#pragma unroll
-    for (int k = 0; k < K; ++k) part[(size_t)blockIdx.x * kMaxMoments + k] = v[k];
-  }
+  block_reduce<K, MAXMASK>(v, red_sm, [&](int k, Acc t) {
+    part[(size_t)blockIdx.x * kMaxMoments + k] = t;
+    __threadfence();  // before thread 0 arrives at the barrier for the block
+  });
   if (!grid_sync(P)) return false;
-  Acc w[K];
-  sum_partials<K, MAXMASK>(part, (int)gridDim.x, w);
-  block_reduce<K, MAXMASK>(w, red_sm);
-  totals<K, Moments<ROLE>::W>(w, P.hx.weight, tot);
+  sum_partials<K, MAXMASK>([&](int k) { return part + k; }, [&](int) { return (int)gridDim.x; }, red_sm,
+                           [&](int k, Acc t) { tot[k] = total<Moments<ROLE>::W>(t, P.hx.weight, k); });
   __syncthreads();
   parity ^= 1;
   return true;
