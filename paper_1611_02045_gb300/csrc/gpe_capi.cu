@@ -47,6 +47,15 @@ struct PrecBufs {
   void* r_prev = nullptr;
 };
 
+// Page-locked landing place of the device's small results: an asynchronous copy
+// to ordinary memory is staged by the driver and takes about 10 us longer.
+struct Pinned {
+  Ctl ctl;
+  AdjScalars adj;
+  TfState tf;
+  VCheck v;
+};
+
 std::string g_create_error;
 
 }  // namespace
@@ -74,6 +83,8 @@ struct gpe_ctx {
   int hflow_cap = 0;
   int hbatch_E = 8;      // values per thread of gpe_apply_H_batch's cluster kernel (plan mode 3):
                          // 16 (streaming form) by default in single precision for n >= 64
+  Pinned* pinned = nullptr;
+  VCheck* vcheck = nullptr;  // extremes of V (device)
   double vmax = 0.0;  // max V on the grid
   double vmin = 0.0;  // min V on the grid
   TfState* tf_state = nullptr;  // Thomas-Fermi root search (device)
@@ -229,41 +240,42 @@ static cudaError_t upload_tables(gpe_ctx* c, PrecBufs& b) {
   return cudaSuccess;
 }
 
-// V of one precision (float32, float64 or double-single) from a device float64
-// copy; the buffer is already allocated.
-static gpe_status upload_V(gpe_ctx* c, int prec, const double* Vdev64) {
-  PrecBufs& b = c->pb[prec];
-  if (prec == 2) GPE_CU(c, launch_d2ds(Vdev64, b.V, c->N, 0));
-  else if (prec == 1) GPE_CU(c, cudaMemcpy(b.V, Vdev64, 8 * (size_t)c->N, cudaMemcpyDeviceToDevice));
-  else GPE_CU(c, launch_d2f(Vdev64, (float*)b.V, c->N, 0));
-  GPE_CU(c, cudaDeviceSynchronize());
+// Take the potential V (float64, host or device): check that it is finite, record
+// its extremes and write it in every precision in use (float32, float64,
+// double-single).  A potential that is not finite changes nothing.  Two kernels on
+// the legacy default stream, which orders them after the caller's work on blocking
+// streams as a plain copy would be, and one host synchronisation: V may be changed
+// or freed when this returns.  The check reads V once and the conversion once more
+// (from L2), where a copy to the host, a loop over it and an allocation took most
+// of a set_problem call (complex128 contexts: 256^2 104 -> 30 us, 128^3 2529 -> 37 us).
+static bool readable_here(const double* p) {  // by a kernel: this device's own memory, aligned
+  cudaPointerAttributes at{};
+  int dev = -1;
+  if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return at.type == cudaMemoryTypeDevice && at.device == dev && (reinterpret_cast<uintptr_t>(p) & 7u) == 0;
+}
+static gpe_status load_V(gpe_ctx* c, const double* V) {
+  const double* src = V;
+  if (!readable_here(V)) {
+    GPE_CU(c, cudaMemcpy(c->pb[1].t, V, 8 * (size_t)c->N, cudaMemcpyDefault));  // a work field as staging
+    src = static_cast<const double*>(c->pb[1].t);
+  }
+  GPE_CU(c, launch_check_V(src, c->N, c->vcheck, 0));
+  GPE_CU(c, launch_take_V(src, c->N, c->vcheck, static_cast<double*>(c->pb[1].V), static_cast<float*>(c->pb[0].V),
+                          c->pb[2].V, 0));
+  GPE_CU(c, cudaMemcpyAsync(&c->pinned->v, c->vcheck, sizeof(VCheck), cudaMemcpyDeviceToHost, 0));
+  GPE_CU(c, cudaStreamSynchronize(0));
+  const VCheck& v = c->pinned->v;
+  if (v.bad) { c->err = "V must be finite"; return GPE_ERR_ARG; }
+  c->vmin = vcheck_value(v.lo);
+  c->vmax = vcheck_value(v.hi);
   return GPE_OK;
 }
 
-// Copy V (float64, host or device) to a new device buffer, check that it is
-// finite and record its maximum (used by the single-precision floor estimate).
-static gpe_status load_V(gpe_ctx* c, const double* V, double** V64_out) {
-  *V64_out = nullptr;
-  double* V64 = nullptr;
-  if (cudaMalloc(&V64, 8 * (size_t)c->N) != cudaSuccess) { c->err = "cudaMalloc V"; return GPE_ERR_CUDA; }
-  std::vector<double> Vh((size_t)c->N);
-  if (cudaMemcpy(V64, V, 8 * (size_t)c->N, cudaMemcpyDefault) != cudaSuccess ||
-      cudaMemcpy(Vh.data(), V64, 8 * (size_t)c->N, cudaMemcpyDeviceToHost) != cudaSuccess) {
-    cudaFree(V64); c->err = "copy of V failed"; return GPE_ERR_CUDA;
-  }
-  double vm = -1e300, vn = 1e300;
-  for (double v : Vh) {
-    if (!std::isfinite(v)) { cudaFree(V64); c->err = "V must be finite"; return GPE_ERR_ARG; }
-    vm = v > vm ? v : vm;
-    vn = v < vn ? v : vn;
-  }
-  c->vmax = vm;
-  c->vmin = vn;
-  *V64_out = V64;
-  return GPE_OK;
-}
-
-static gpe_status alloc_prec(gpe_ctx* c, int prec, const double* Vdev64) {
+static gpe_status alloc_prec(gpe_ctx* c, int prec) {
   PrecBufs& b = c->pb[prec];
   b.on = true;
   const size_t cb = prec ? 16 : 8;  // complex64 8 B; complex128 and double-single 16 B
@@ -278,7 +290,7 @@ static gpe_status alloc_prec(gpe_ctx* c, int prec, const double* Vdev64) {
   GPE_CU(c, cudaMemset(b.p, 0, bytes));
   GPE_CU(c, cudaMemset(b.r_prev, 0, bytes));
   GPE_CU(c, cudaMalloc(&b.V, (prec == 0 ? 4 : 8) * (size_t)c->N));
-  return upload_V(c, prec, Vdev64);
+  return GPE_OK;
 }
 
 static void free_ctx(gpe_ctx* c) {
@@ -291,6 +303,8 @@ static void free_ctx(gpe_ctx* c) {
   cudaFree(c->pers_partials); cudaFree(c->pers_bar);
   for (auto& a : c->adj) cudaFree(a);
   cudaFree(c->tf_state);
+  cudaFree(c->vcheck);
+  if (c->pinned) cudaFreeHost(c->pinned);
   cudaFree(c->adj_s); cudaFree(c->adj_partials);
   cudaFree(c->hflow_ctr);
   cudaFree(c->ctl_solve); cudaFree(c->ctl_api); cudaFree(c->partials); cudaFree(c->ticket); cudaFree(c->log_dev);
@@ -346,16 +360,14 @@ extern "C" gpe_status gpe_create(const gpe_problem* prob, const double* V, void*
   auto fail = [&](gpe_status s) { g_create_error = c->err; free_ctx(c); return s; };
   if (cudaStreamCreateWithFlags(&c->cap, cudaStreamNonBlocking) != cudaSuccess) { c->err = "stream create failed"; return fail(GPE_ERR_CUDA); }
 
-  // potential: a device float64 copy is the source of every precision
-  double* V64 = nullptr;
-  {
-    const gpe_status sv = load_V(c, V, &V64);
-    if (sv != GPE_OK) return fail(sv);
+  gpe_status s = alloc_prec(c, 1);
+  if (s == GPE_OK && prob->prec == GPE_MIXED) s = alloc_prec(c, 0);
+  if (s == GPE_OK && prob->prec == GPE_MIXED) s = alloc_prec(c, 2);
+  if (s != GPE_OK) return fail(s);
+  if (cudaMalloc(&c->vcheck, sizeof(VCheck)) != cudaSuccess || cudaMallocHost(&c->pinned, sizeof(Pinned)) != cudaSuccess) {
+    c->err = "cudaMalloc workspace"; return fail(GPE_ERR_CUDA);
   }
-  gpe_status s = alloc_prec(c, 1, V64);
-  if (s == GPE_OK && prob->prec == GPE_MIXED) s = alloc_prec(c, 0, V64);
-  if (s == GPE_OK && prob->prec == GPE_MIXED) s = alloc_prec(c, 2, V64);
-  cudaFree(V64);
+  s = load_V(c, V);
   if (s != GPE_OK) return fail(s);
 
   int maxblocks = 1;
@@ -516,9 +528,9 @@ extern "C" gpe_status gpe_energy(gpe_ctx* c, const void* phi, double out[8]) {
   const int prec = c->work;
   gpe_status s = run_H(c, prec, phi, phi, c->pb[prec].t, c->ctl_api);
   if (s != GPE_OK) return s;
-  Ctl h;
-  GPE_CU(c, cudaMemcpyAsync(&h, c->ctl_api, sizeof(Ctl), cudaMemcpyDeviceToHost, c->st));
+  GPE_CU(c, cudaMemcpyAsync(&c->pinned->ctl, c->ctl_api, sizeof(Ctl), cudaMemcpyDeviceToHost, c->st));
   GPE_CU(c, cudaStreamSynchronize(c->st));
+  const Ctl& h = c->pinned->ctl;
   out[0] = h.kin; out[1] = h.pot; out[2] = 0.5 * c->prob.eta * h.U0; out[3] = h.rot;
   out[4] = h.E; out[5] = h.lam; out[6] = h.alpha; out[7] = h.norm2;
   return GPE_OK;
@@ -529,12 +541,7 @@ extern "C" gpe_status gpe_set_problem(gpe_ctx* c, const double* V, double eta, d
   if (!std::isfinite(eta) || !std::isfinite(omega)) { c->err = "eta/omega must be finite"; return GPE_ERR_ARG; }
   GPE_CU(c, cudaStreamSynchronize(c->st));
   if (V) {
-    double* V64 = nullptr;
-    gpe_status s = load_V(c, V, &V64);
-    if (s != GPE_OK) return s;
-    for (int prec = 0; prec < 3 && s == GPE_OK; ++prec)
-      if (c->pb[prec].on) s = upload_V(c, prec, V64);
-    cudaFree(V64);
+    const gpe_status s = load_V(c, V);
     if (s != GPE_OK) return s;
   }
   c->prob.eta = eta;
@@ -556,9 +563,9 @@ extern "C" gpe_status gpe_energy_grad(gpe_ctx* c, const void* phi, void* grad_ph
   gpe_status s = run_H(c, prec, phi, phi, hphi, c->ctl_api);
   if (s != GPE_OK) return s;
   if (grad_phi || grad_V) GPE_CU(c, launch_grad_epilogue(prec, phi, grad_phi, grad_V, c->N, c->weight, c->st));
-  Ctl h;
-  GPE_CU(c, cudaMemcpyAsync(&h, c->ctl_api, sizeof(Ctl), cudaMemcpyDeviceToHost, c->st));
+  GPE_CU(c, cudaMemcpyAsync(&c->pinned->ctl, c->ctl_api, sizeof(Ctl), cudaMemcpyDeviceToHost, c->st));
   GPE_CU(c, cudaStreamSynchronize(c->st));
+  const Ctl& h = c->pinned->ctl;
   out[0] = h.E;
   out[1] = 0.5 * h.U0;  // d/d eta of eta/2 int |phi|^4
   out[2] = -h.Lz;       // d/d omega of -omega <phi, L_z phi>
@@ -593,8 +600,9 @@ extern "C" gpe_status gpe_thomas_fermi(gpe_ctx* c, void* phi_out, double* mu_out
     for (int k = 0; k < kTfCheck; ++k)
       GPE_CU(c, launch_tf_step(V64, c->N, c->weight / c->prob.eta, c->tf_state, init, it + k == 0, c->partials,
                                c->ticket, c->st));
-    GPE_CU(c, cudaMemcpyAsync(&S, c->tf_state, sizeof(S), cudaMemcpyDeviceToHost, c->st));
+    GPE_CU(c, cudaMemcpyAsync(&c->pinned->tf, c->tf_state, sizeof(S), cudaMemcpyDeviceToHost, c->st));
     GPE_CU(c, cudaStreamSynchronize(c->st));
+    S = c->pinned->tf;
   }
   const bool dev = is_device_ptr(phi_out);
   void* dst = dev ? phi_out : c->pb[1].phi;
@@ -726,10 +734,9 @@ static gpe_status tangent_solve(gpe_ctx* c, const void* phi, const void* rhs, vo
   // lambda = <phi, H phi> and the shift lambda~ of eq. Opt_Alpha at phi
   gpe_status s = run_H(c, prec, phi, phi, q, c->ctl_api);
   if (s != GPE_OK) return s;
-  Ctl h;
-  GPE_CU(c, cudaMemcpyAsync(&h, c->ctl_api, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
+  GPE_CU(c, cudaMemcpyAsync(&c->pinned->ctl, c->ctl_api, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
   GPE_CU(c, cudaStreamSynchronize(st));
-  const double lam = h.lam, alpha = h.alpha;
+  const double lam = c->pinned->ctl.lam, alpha = c->pinned->ctl.alpha;
   if (!std::isfinite(lam) || !(alpha > 0.0)) { c->err = "phi gives a non-finite lambda or a shift <= 0"; return GPE_ERR_NONFINITE; }
   AdjScalars s0;
   std::memset(&s0, 0, sizeof(s0));
@@ -751,8 +758,9 @@ static gpe_status tangent_solve(gpe_ctx* c, const void* phi, const void* rhs, vo
   int it = 0;
   for (;;) {
     if (it % kAdjCheckEvery == 0 || it >= max_iter) {
-      GPE_CU(c, cudaMemcpyAsync(&hs, S, sizeof(hs), cudaMemcpyDeviceToHost, st));
+      GPE_CU(c, cudaMemcpyAsync(&c->pinned->adj, S, sizeof(hs), cudaMemcpyDeviceToHost, st));
       GPE_CU(c, cudaStreamSynchronize(st));
+      hs = c->pinned->adj;
       if (hs.stop || it >= max_iter) break;
     }
     // q = P K p;  a = Re<r, y> / Re<p, q>;  z += a p;  r -= a q
@@ -1044,11 +1052,12 @@ static gpe_status run_phase(gpe_ctx* c, int mode, Ctl& h, const gpe_solve_opts& 
       }
     }
   }
-  GPE_CU(c, cudaMemcpyAsync(&h, c->ctl_solve, sizeof(Ctl), cudaMemcpyDeviceToHost, c->st));
+  GPE_CU(c, cudaMemcpyAsync(&c->pinned->ctl, c->ctl_solve, sizeof(Ctl), cudaMemcpyDeviceToHost, c->st));
   int wait_failed = 0;
   if (loop == 2)  // a barrier wait of the persistent kernel gave up (any block)
     GPE_CU(c, cudaMemcpyAsync(&wait_failed, c->pers_bar + 2, sizeof(int), cudaMemcpyDeviceToHost, c->st));
   GPE_CU(c, cudaStreamSynchronize(c->st));
+  h = c->pinned->ctl;
   if (wait_failed) {
     h.status = GPE_ERR_TIMEOUT;
     h.done = 1;

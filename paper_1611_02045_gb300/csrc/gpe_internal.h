@@ -221,8 +221,23 @@ cudaError_t launch_cluster_solve(int M, const ClusterSolveArgs& P, cudaStream_t 
 // Small elementwise/control kernels (gpe_misc.cu).
 cudaError_t launch_convert_c128_to_c64(const void* src, void* dst, long long n, cudaStream_t st);
 cudaError_t launch_convert_c64_to_c128(const void* src, void* dst, long long n, cudaStream_t st);
-cudaError_t launch_d2f(const double* src, float* dst, long long n, cudaStream_t st);
-cudaError_t launch_d2ds(const double* src, void* dst, long long n, cudaStream_t st);
+// Extremes of a potential, as keys that order like the doubles they stand for, and
+// whether any value is not finite.
+struct VCheck {
+  long long lo, hi;
+  int bad, pad;
+};
+inline double vcheck_value(long long key) {
+  const long long b = key < 0 ? (key ^ 0x7fffffffffffffffll) : key;
+  double v;
+  static_assert(sizeof(v) == sizeof(b), "64-bit doubles");
+  __builtin_memcpy(&v, &b, sizeof(v));
+  return v;
+}
+cudaError_t launch_check_V(const double* V, long long n, VCheck* out, cudaStream_t st);
+// V in float64, float32 and double-single (null outputs are skipped); nothing when check->bad.
+cudaError_t launch_take_V(const double* V, long long n, const VCheck* check, double* v64, float* v32, void* vds,
+                          cudaStream_t st);
 cudaError_t launch_convert_c64_to_ds(const void* src, void* dst, long long n, cudaStream_t st);
 cudaError_t launch_convert_ds_to_c128(const void* src, void* dst, long long n, cudaStream_t st);
 // ctl->cc = 1 / ||phi||, ss = 0, retract = 1 (weighted norm), so that the next

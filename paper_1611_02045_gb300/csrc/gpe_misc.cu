@@ -80,11 +80,6 @@ __global__ void k_c64_to_c128(const float2* __restrict__ s, double2* __restrict_
     d[i] = make_double2((double)v.x, (double)v.y);
   }
 }
-__global__ void k_d2f(const double* __restrict__ s, float* __restrict__ d, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    d[i] = (float)s[i];
-}
-
 // double-single <-> complex64 / complex128 (the refinement state)
 __global__ void k_c64_to_ds(const float2* __restrict__ s, dsc* __restrict__ d, long long n) {
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
@@ -123,16 +118,54 @@ cudaError_t launch_convert_ds_to_c128(const void* src, void* dst, long long n, c
   k_ds_to_c128<<<grid_for(n), 256, 0, st>>>((const dsc*)src, (double2*)dst, n);
   return cudaGetLastError();
 }
-__global__ void k_d2ds(const double* __restrict__ s, dsf* __restrict__ d, long long n) {
-  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-    d[i] = dsf(s[i]);
+// Extremes and finiteness of V on the integer pipe: the bits of a double, negative
+// ones with the magnitude inverted, order like the values.
+__device__ __forceinline__ long long order_key(long long b) { return b ^ ((b >> 63) & 0x7fffffffffffffffll); }
+__global__ void k_check_init(VCheck* out) {
+  out->lo = 0x7fffffffffffffffll;
+  out->hi = -0x7fffffffffffffffll - 1;
+  out->bad = 0;
 }
-cudaError_t launch_d2ds(const double* src, void* dst, long long n, cudaStream_t st) {
-  k_d2ds<<<grid_for(n), 256, 0, st>>>(src, (dsf*)dst, n);
+__global__ void __launch_bounds__(256) k_check_V(const double* __restrict__ V, long long n, VCheck* out) {
+  long long lo = 0x7fffffffffffffffll, hi = -lo - 1;
+  int bad = 0;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const long long b = __double_as_longlong(V[i]), k = order_key(b);
+    bad |= (b & 0x7ff0000000000000ll) == 0x7ff0000000000000ll;
+    lo = k < lo ? k : lo;
+    hi = k > hi ? k : hi;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    const long long l2 = __shfl_xor_sync(0xffffffffu, lo, o), h2 = __shfl_xor_sync(0xffffffffu, hi, o);
+    lo = l2 < lo ? l2 : lo;
+    hi = h2 > hi ? h2 : hi;
+  }
+  bad = __any_sync(0xffffffffu, bad);
+  if ((threadIdx.x & 31) == 0) {
+    atomicMin(&out->lo, lo);
+    atomicMax(&out->hi, hi);
+    if (bad) atomicOr(&out->bad, 1);
+  }
+}
+cudaError_t launch_check_V(const double* V, long long n, VCheck* out, cudaStream_t st) {
+  k_check_init<<<1, 1, 0, st>>>(out);
+  const int g = grid_for(n);
+  k_check_V<<<g < 608 ? g : 608, 256, 0, st>>>(V, n, out);
   return cudaGetLastError();
 }
-cudaError_t launch_d2f(const double* src, float* dst, long long n, cudaStream_t st) {
-  k_d2f<<<grid_for(n), 256, 0, st>>>(src, dst, n);
+__global__ void k_take_V(const double* __restrict__ V, long long n, const VCheck* __restrict__ check,
+                         double* __restrict__ v64, float* __restrict__ v32, dsf* __restrict__ vds) {
+  if (check->bad) return;
+  for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const double v = V[i];
+    if (v64) v64[i] = v;
+    if (v32) v32[i] = (float)v;
+    if (vds) vds[i] = dsf(v);
+  }
+}
+cudaError_t launch_take_V(const double* V, long long n, const VCheck* check, double* v64, float* v32, void* vds,
+                          cudaStream_t st) {
+  k_take_V<<<grid_for(n), 256, 0, st>>>(V, n, check, v64, v32, (dsf*)vds);
   return cudaGetLastError();
 }
 
