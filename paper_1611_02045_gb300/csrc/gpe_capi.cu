@@ -419,8 +419,13 @@ extern "C" const char* gpe_last_error(const gpe_ctx* c) { return c ? c->err.c_st
 
 // H passes on (phi, f): t = A_x f + (V + eta|phi|^2) f, then the y (and z) parts
 // accumulated; the last one writes `out` (or t) and finalises the energy terms.
-// moments = false: H phi as a plain operator (gpe_apply_H); the passes skip the
-// energy moments and the scalar step that only gpe_energy and the solver read.
+// H_ONLY: H phi as a plain operator (gpe_apply_H); the passes skip the energy
+// moments and the scalar step that only gpe_energy and the solver read.
+// MOMENTS_ONLY: the energy terms of phi (f = phi; f, out and t are not touched):
+// forward transforms alone, 8 + 4 and 8 bytes per point and pass instead of 20 and 24
+// (complex64; P_C r with its own shift on 256 x 128 x 64: 116 -> 106 us; gpe_energy in
+// complex128: 128^3 797 -> 355 us with the shorter FP64 passes).
+enum HWant { H_AND_MOMENTS, H_ONLY, MOMENTS_ONLY };
 // The x and y parts of H phi on complex64 planes as a dataflow (gpe_hflow.cu):
 // nplanes planes of the context's nx x ny, V one plane (vstride 0) or one per plane.
 // The dataflow needs enough units to fill its pipeline (a unit is 4096 points, 304
@@ -465,15 +470,16 @@ static gpe_status try_flow(gpe_ctx* c, int nplanes, long long vstride, const voi
 }
 
 static gpe_status run_H(gpe_ctx* c, int prec, const void* phi, const void* f, void* out, Ctl* ctl,
-                        bool moments = true) {
+                        HWant want = H_AND_MOMENTS) {
   bool flowed = false;
-  if (prec == 0 && !moments && c->dim == 3 && flow_pays(c, c->N)) {
+  if (prec == 0 && want == H_ONLY && c->dim == 3 && flow_pays(c, c->N)) {
     const gpe_status s = try_flow(c, c->n[2], (long long)c->n[0] * c->n[1], phi, f, c->pb[0].t, &flowed);
     if (s != GPE_OK) return s;
   }
   PassArgs a = base_args(c, prec, 0, prec);
   a.ctl = ctl; a.phi = phi; a.f = f; a.t = c->pb[prec].t;
-  a.nomoments = moments ? 0 : 1;
+  a.nomoments = want == H_ONLY ? 1 : 0;
+  a.eonly = want == MOMENTS_ONLY ? 1 : 0;
   // fields above 64 MB (beyond L2 with the operator's other arrays): the x pass
   // prefetches the rows of the block one wave ahead (two blocks per SM)
   if ((double)c->N * (prec == 0 ? 8.0 : 16.0) > 64.0 * 1024 * 1024) a.pf = 2 * c->nsm;
@@ -482,6 +488,7 @@ static gpe_status run_H(gpe_ctx* c, int prec, const void* phi, const void* f, vo
     PassArgs b = base_args(c, prec, ax, prec);
     b.ctl = ctl; b.phi = phi; b.f = f; b.t = c->pb[prec].t;
     b.nomoments = a.nomoments;
+    b.eonly = a.eonly;
     b.last_axis = (ax == c->dim - 1);
     b.out = b.last_axis ? out : nullptr;
     GPE_CU(c, launch(prec, P_HMID, b, c->st));
@@ -492,7 +499,7 @@ static gpe_status run_H(gpe_ctx* c, int prec, const void* phi, const void* f, vo
 extern "C" gpe_status gpe_apply_H(gpe_ctx* c, const void* phi, const void* f, void* out) {
   if (!c) return GPE_ERR_ARG;
   if (!phi || !f || !out) { c->err = "null field pointer"; return GPE_ERR_ARG; }
-  return run_H(c, c->work, phi, f, out, c->ctl_api, false);
+  return run_H(c, c->work, phi, f, out, c->ctl_api, H_ONLY);
 }
 
 extern "C" gpe_status gpe_apply_H_batch(gpe_ctx* c, int nbatch, const void* phi, const void* f, void* out) {
@@ -526,7 +533,7 @@ extern "C" gpe_status gpe_energy(gpe_ctx* c, const void* phi, double out[8]) {
   if (!c) return GPE_ERR_ARG;
   if (!phi || !out) { c->err = "null pointer"; return GPE_ERR_ARG; }
   const int prec = c->work;
-  gpe_status s = run_H(c, prec, phi, phi, c->pb[prec].t, c->ctl_api);
+  gpe_status s = run_H(c, prec, phi, phi, nullptr, c->ctl_api, MOMENTS_ONLY);
   if (s != GPE_OK) return s;
   GPE_CU(c, cudaMemcpyAsync(&c->pinned->ctl, c->ctl_api, sizeof(Ctl), cudaMemcpyDeviceToHost, c->st));
   GPE_CU(c, cudaStreamSynchronize(c->st));
@@ -559,8 +566,7 @@ extern "C" gpe_status gpe_energy_grad(gpe_ctx* c, const void* phi, void* grad_ph
   if (!phi || !out) { c->err = "null pointer"; return GPE_ERR_ARG; }
   if (grad_phi == phi) { c->err = "grad_phi must not overlap phi"; return GPE_ERR_ARG; }
   const int prec = c->work;
-  void* hphi = grad_phi ? grad_phi : c->pb[prec].t;
-  gpe_status s = run_H(c, prec, phi, phi, hphi, c->ctl_api);
+  gpe_status s = run_H(c, prec, phi, phi, grad_phi, c->ctl_api, grad_phi ? H_AND_MOMENTS : MOMENTS_ONLY);
   if (s != GPE_OK) return s;
   if (grad_phi || grad_V) GPE_CU(c, launch_grad_epilogue(prec, phi, grad_phi, grad_V, c->N, c->weight, c->st));
   GPE_CU(c, cudaMemcpyAsync(&c->pinned->ctl, c->ctl_api, sizeof(Ctl), cudaMemcpyDeviceToHost, c->st));
@@ -706,7 +712,7 @@ extern "C" gpe_status gpe_precond(gpe_ctx* c, const void* phi, const void* r, do
   if (!std::isfinite(alpha)) { c->err = "alpha must be finite"; return GPE_ERR_ARG; }
   const int prec = c->work;
   if (!(alpha > 0.0)) {
-    gpe_status s = run_H(c, prec, phi, phi, c->pb[prec].t, c->ctl_api);  // lambda~ into ctl_api->alpha
+    gpe_status s = run_H(c, prec, phi, phi, nullptr, c->ctl_api, MOMENTS_ONLY);  // lambda~ into ctl_api->alpha
     if (s != GPE_OK) return s;
   }
   IterBufs b = iter_bufs(c, prec);
@@ -732,7 +738,7 @@ static gpe_status tangent_solve(gpe_ctx* c, const void* phi, const void* rhs, vo
   const double w = c->weight;
   cudaStream_t st = c->st;
   // lambda = <phi, H phi> and the shift lambda~ of eq. Opt_Alpha at phi
-  gpe_status s = run_H(c, prec, phi, phi, q, c->ctl_api);
+  gpe_status s = run_H(c, prec, phi, phi, nullptr, c->ctl_api, MOMENTS_ONLY);
   if (s != GPE_OK) return s;
   GPE_CU(c, cudaMemcpyAsync(&c->pinned->ctl, c->ctl_api, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
   GPE_CU(c, cudaStreamSynchronize(st));
@@ -764,7 +770,7 @@ static gpe_status tangent_solve(gpe_ctx* c, const void* phi, const void* rhs, vo
       if (hs.stop || it >= max_iter) break;
     }
     // q = P K p;  a = Re<r, y> / Re<p, q>;  z += a p;  r -= a q
-    if ((s = run_H(c, prec, phi, p, q, c->ctl_api, false)) != GPE_OK) return s;
+    if ((s = run_H(c, prec, phi, p, q, c->ctl_api, H_ONLY)) != GPE_OK) return s;
     GPE_CU(c, adj_hess_epi(prec, phi, p, q, N, c->prob.eta, lam, w, aw, st));
     GPE_CU(c, adj_step(prec, z, r, p, q, phi, N, w, aw, st));
     // y = P_C r;  beta = Re<r, P y> / previous;  p = P y + beta p

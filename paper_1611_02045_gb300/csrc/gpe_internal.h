@@ -123,6 +123,8 @@ struct PassArgs {
   int pf;          // contiguous H pass outside a solve: L2 prefetch of the rows of unit + pf (0: none)
   int solver;      // 1: inside a solve (uses ctl scalars, solver reductions)
   int nomoments;   // 1: the caller needs no reductions (H phi as a plain operator): passes skip them
+  int eonly;       // 1: only the energy moments are wanted (gpe_energy, the shift of P_C): the H passes stop
+                   // after their forward transforms and write no field
   int last_axis;   // 1: this pass is the final one of its operator (runs the finaliser)
   double weight;   // h^d
   double eta, omega;

@@ -58,7 +58,8 @@ __global__ void __launch_bounds__(512) pass_s_tma(PassArgs a, const __grid_const
   C* ex = stage + 2 * NT * tile;           // transform exchange [M][tx]
   const int c = threadIdx.x % tx, t = threadIdx.x / tx;
   const long long units = a.nblocks;
-  const unsigned bytes = (unsigned)NT * (unsigned)tile * (unsigned)sizeof(C);
+  const bool two = NT == 2 && !a.eonly;  // the energy moments need no accumulated t
+  const unsigned bytes = (two ? 2u : 1u) * (unsigned)tile * (unsigned)sizeof(C);
 
   if (threadIdx.x == 0) {
     mbar_init(&bar[0], 1);
@@ -80,7 +81,7 @@ __global__ void __launch_bounds__(512) pass_s_tma(PassArgs a, const __grid_const
       const int y0 = a.axis == 1 ? b * BOX : outer;
       const int z0 = a.axis == 1 ? outer : b * BOX;
       tma_load_3d(d0 + b * BOX * tx, &tm0, x0, y0, z0, &bar[s]);
-      if constexpr (NT == 2) tma_load_3d(d0 + tile + b * BOX * tx, &tm1, x0, y0, z0, &bar[s]);
+      if (two) tma_load_3d(d0 + tile + b * BOX * tx, &tm1, x0, y0, z0, &bar[s]);
     }
   };
 
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(512) pass_s_tma(PassArgs a, const __grid_const
       // t += (1/2 mu^2 - omega x mu) f (y) or 1/2 zeta^2 f (z), the operand tile, then t
       C tv[E];
 #pragma unroll
-      for (int q = 0; q < E; ++q) tv[q] = in0[tile + (t + q * Tl) * tx + c];
+      for (int q = 0; q < E; ++q) tv[q] = two ? in0[tile + (t + q * Tl) * tx + c] : make_float2(0.0f, 0.0f);
       line_dft<M, E, -1>(v, ex, si, t, tw);
       const T rx = (a.axis == 1) ? -tab<T>(a.xc[0])[ix] : T(0);  // rotation symbol -omega x mu (y); none for z
       if (!a.nomoments) {
@@ -133,11 +134,13 @@ __global__ void __launch_bounds__(512) pass_s_tma(PassArgs a, const __grid_const
         acc[0] = acc_add(acc[0], acc_from(T(0.5) * s2 * invM));
         acc[1] = acc_add(acc[1], acc_from(rx * s1 * invM));
       }
-      apply_symbol<E>(v, xia, t, Tl, T(0.5) * invM, om * rx * invM);
-      line_dft<M, E, +1>(v, ex, si, t, tw);
-      C* __restrict__ dst = static_cast<C*>(a.out ? a.out : a.t);  // API: the final pass writes the caller's buffer
+      if (!a.eonly) {
+        apply_symbol<E>(v, xia, t, Tl, T(0.5) * invM, om * rx * invM);
+        line_dft<M, E, +1>(v, ex, si, t, tw);
+        C* __restrict__ dst = static_cast<C*>(a.out ? a.out : a.t);  // API: the final pass writes the caller's buffer
 #pragma unroll
-      for (int q = 0; q < E; ++q) dst[base + (t + q * Tl) * a.stride] = cadd(tv[q], v[q]);
+        for (int q = 0; q < E; ++q) dst[base + (t + q * Tl) * a.stride] = cadd(tv[q], v[q]);
+      }
     } else if constexpr (ROLE == P_CFWD || ROLE == P_CINV || ROLE == P_CCORE) {
       if constexpr (ROLE == P_CINV) {
         line_dft<M, E, +1>(v, ex, si, t, tw);
@@ -288,14 +291,16 @@ __global__ void __launch_bounds__(512) pass_hx_bulk(PassArgs a, int second) {
       acc[0] = acc_add(acc[0], acc_from(T(0.5) * s2 * invM));
       acc[1] = acc_add(acc[1], acc_from(y * s1 * invM));
     }
-    apply_symbol<E>(v, xi, t, Tl, T(0.5) * invM, om * y * invM);
-    line_dft<M, E, +1, W>(v, sm, si, t, tw);
+    if (!a.eonly) {
+      apply_symbol<E>(v, xi, t, Tl, T(0.5) * invM, om * y * invM);
+      line_dft<M, E, +1, W>(v, sm, si, t, tw);
 #pragma unroll
-    for (int q = 0; q < E; ++q) {
-      const T uu = ph[q].x * ph[q].x + ph[q].y * ph[q].y;
-      const T m = vv[q] + eta * uu;
-      const C fq = (second == 1) ? secs[q * Tl] : ph[q];  // the operand f (API call with f != phi)
-      tout[base + q * Tl] = make_float2(v[q].x + m * fq.x, v[q].y + m * fq.y);
+      for (int q = 0; q < E; ++q) {
+        const T uu = ph[q].x * ph[q].x + ph[q].y * ph[q].y;
+        const T m = vv[q] + eta * uu;
+        const C fq = (second == 1) ? secs[q * Tl] : ph[q];  // the operand f (API call with f != phi)
+        tout[base + q * Tl] = make_float2(v[q].x + m * fq.x, v[q].y + m * fq.y);
+      }
     }
     if (!a.nomoments) {
       T apot = 0, au2 = 0, an2 = 0, umax = 0;

@@ -751,17 +751,19 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
       acc[0] = acc_add(acc[0], acc_from(TF(0.5) * s2 * invM));
       acc[1] = acc_add(acc[1], acc_from(y * s1 * invM));
     }
-    apply_symbol<E>(v, xi, t, Tl, TF(0.5) * invM, num_as<TF>(a.omega_n) * y * invM);
-    line_dft<M, E, +1, W>(v, sm, si, t, tw);
-    CS* __restrict__ tout = static_cast<CS*>(a.t);
-    const TS eta = num_as<TS>(a.eta_n);
+    if (!a.eonly) {  // uniform
+      apply_symbol<E>(v, xi, t, Tl, TF(0.5) * invM, num_as<TF>(a.omega_n) * y * invM);
+      line_dft<M, E, +1, W>(v, sm, si, t, tw);
+      CS* __restrict__ tout = static_cast<CS*>(a.t);
+      const TS eta = num_as<TS>(a.eta_n);
 #pragma unroll
-    for (int q = 0; q < E; ++q) {
-      const long long g = base + t + q * Tl;
-      const TS u = ph[q].x * ph[q].x + ph[q].y * ph[q].y;
-      const TS m = vv[q] + eta * u;
-      const CS fq = (a.f && !a.solver) ? f[g] : ph[q];  // the operand f (re-read in API mode)
-      tout[g] = cmk<CS>(TS(v[q].x) + m * fq.x, TS(v[q].y) + m * fq.y);
+      for (int q = 0; q < E; ++q) {
+        const long long g = base + t + q * Tl;
+        const TS u = ph[q].x * ph[q].x + ph[q].y * ph[q].y;
+        const TS m = vv[q] + eta * u;
+        const CS fq = (a.f && !a.solver) ? f[g] : ph[q];  // the operand f (re-read in API mode)
+        tout[g] = cmk<CS>(TS(v[q].x) + m * fq.x, TS(v[q].y) + m * fq.y);
+      }
     }
     if (!a.nomoments) {
       TS apot = 0, au2 = 0, an2 = 0, umax = 0;
@@ -946,7 +948,7 @@ __device__ __forceinline__ void sunit(const PassArgs& a, const Scal& S, long lon
 #pragma unroll
     for (int q = 0; q < E; ++q) {
       v[q] = f[base + (t + q * Tl) * st];
-      tv[q] = tb[base + (t + q * Tl) * st];
+      if (!a.eonly) tv[q] = tb[base + (t + q * Tl) * st];
     }
     if (S.done) return;
     line_dft<M, E, -1>(v, sm, si, t, tw);
@@ -957,6 +959,7 @@ __device__ __forceinline__ void sunit(const PassArgs& a, const Scal& S, long lon
       acc[0] = acc_add(acc[0], acc_from(T(0.5) * s2 * invM));
       acc[1] = acc_add(acc[1], acc_from(rx * s1 * invM));
     }
+    if (a.eonly) return;  // uniform
     apply_symbol<E>(v, xia, t, Tl, T(0.5) * invM, num_as<T>(a.omega_n) * rx * invM);
     line_dft<M, E, +1>(v, sm, si, t, tw);
     C* __restrict__ dst = static_cast<C*>(a.out ? a.out : a.t);  // API: final pass writes the caller's buffer
