@@ -496,9 +496,32 @@ static gpe_status run_H(gpe_ctx* c, int prec, const void* phi, const void* f, vo
   return GPE_OK;
 }
 
+static ClusterHArgs cluster_args(const gpe_ctx* c, int prec, int nbatch, const void* phi, const void* f, void* out) {
+  const PrecBufs& b = c->pb[prec];
+  ClusterHArgs a;
+  std::memset(&a, 0, sizeof(a));
+  a.M = c->n[0]; a.nbatch = nbatch; a.stride = c->N;
+  a.eta = c->prob.eta; a.omega = c->prob.omega;
+  a.xi = b.xi[0]; a.xiy = b.xi[1]; a.xc = b.xc[0]; a.yc = b.xc[1]; a.tw = b.tw[0]; a.V = b.V;
+  a.phi = phi; a.f = f; a.out = out;
+  a.E = c->hbatch_E;
+  a.rows = c->hbatch_rows;
+  return a;
+}
+
 extern "C" gpe_status gpe_apply_H(gpe_ctx* c, const void* phi, const void* f, void* out) {
   if (!c) return GPE_ERR_ARG;
   if (!phi || !f || !out) { c->err = "null field pointer"; return GPE_ERR_ARG; }
+  if (c->work == 0 && c->dim == 2 && c->n[0] == c->n[1] && c->n[0] >= 32 && c->n[0] <= 128) {
+    // one launch for a small square field, in one cluster (which reads all of f before it
+    // writes: out may be f).  Device time against the two passes: 32^2 4.7 / 6.7 us, 64^2
+    // 6.1 / 8.4, 128^2 8.5 / 9.4, 256^2 15.1 / 9.5; in complex128 the FP64 pipes of the
+    // cluster's few SMs are the limit (32^2 27 / 17 us)
+    ClusterHArgs a = cluster_args(c, 0, 1, phi, f, out);
+    a.E = 8;
+    GPE_CU(c, launch_cluster_apply_H(0, a, c->st));
+    return GPE_OK;
+  }
   return run_H(c, c->work, phi, f, out, c->ctl_api, H_ONLY);
 }
 
@@ -511,15 +534,7 @@ extern "C" gpe_status gpe_apply_H_batch(gpe_ctx* c, int nbatch, const void* phi,
   }
   if (nbatch == 0) return GPE_OK;
   const int prec = c->work;
-  const PrecBufs& b = c->pb[prec];
-  ClusterHArgs a;
-  std::memset(&a, 0, sizeof(a));
-  a.M = c->n[0]; a.nbatch = nbatch; a.stride = c->N;
-  a.eta = c->prob.eta; a.omega = c->prob.omega;
-  a.xi = b.xi[0]; a.xiy = b.xi[1]; a.xc = b.xc[0]; a.yc = b.xc[1]; a.tw = b.tw[0]; a.V = b.V;
-  a.phi = phi; a.f = f; a.out = out;
-  a.E = c->hbatch_E;
-  a.rows = c->hbatch_rows;
+  const ClusterHArgs a = cluster_args(c, prec, nbatch, phi, f, out);
   if (prec == 0 && a.E == 16 && a.rows == 16 && flow_pays(c, nbatch * c->N)) {
     bool used = false;
     const gpe_status s = try_flow(c, nbatch, 0, phi, f, out, &used);
