@@ -50,6 +50,16 @@ __device__ __forceinline__ dsf operator*(dsf a, dsf b) {
   e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e));
   return ds_fast_two_sum(p, e);
 }
+// Products with FP32 factors: one rounding less than with a factor whose low part is
+// zero, and two FP32 factors give their product exactly.
+__device__ __forceinline__ dsf ds_mul(dsf a, float b) {
+  const float p = a.hi * b;
+  return ds_fast_two_sum(p, fmaf(a.lo, b, fmaf(a.hi, b, -p)));
+}
+__device__ __forceinline__ dsf ds_mul(float a, float b) {
+  const float p = a * b;
+  return dsf(p, fmaf(a, b, -p));
+}
 __device__ __forceinline__ dsf operator/(dsf a, dsf b) {
   const float q1 = a.hi / b.hi;
   const dsf r = a - b * dsf(q1);

@@ -589,6 +589,20 @@ template <typename T> __device__ __forceinline__ T pv_factor(T den, int code) {
 template <> __device__ __forceinline__ double pv_factor<double>(double den, int code) {
   return code == 0 ? 1.0 : (code == 2 ? __drcp_rn(den) : rsqrt(den));
 }
+// Double-single: the FP32 reciprocal square root with a second-order correction from
+// its residual e = 1 - den y^2 ((1 - e)^{-1/2} = 1 + e/2 + 3 e^2/8 + ..., e ~ 2^-22, so
+// e^3 is below the last bit), about 20 operations where a square root and a division
+// take some 110; relative error against FP64 1.6e-14 at most, 1.9e-15 rms (1.6e-14 and
+// 2.4e-15 with root and division).
+template <> __device__ __forceinline__ dsf pv_factor<dsf>(dsf den, int code) {
+  if (code == 0) return dsf(1.0f);
+  if (code == 2) return dsf(1.0f) / den;
+  const float y = rsqrtf(den.hi);
+  const float th = den.hi * y, tl = fmaf(den.lo, y, fmaf(den.hi, y, -th));  // den y
+  const float p = th * y;
+  const float e = (1.0f - p) - fmaf(tl, y, fmaf(th, y, -p));
+  return ds_fast_two_sum(y, y * e * fmaf(0.375f, e, 0.5f));
+}
 // p / den for a power of two p: FP64 takes the (correctly rounded) reciprocal,
 // whose scaling is exact, in place of the longer division.
 template <typename T> __device__ __forceinline__ T over(T p, T den) { return p / den; }
@@ -611,6 +625,17 @@ __device__ __forceinline__ Scal scal_of(const Ctl* c, const PassArgs& a) {
 // ---------------------------------------------------------------------------
 template <typename T>
 __device__ __forceinline__ const T* tab(const void* p) { return static_cast<const T*>(p); }
+
+// Products of a state value with a direction value, and of two direction values, in
+// the state's type.
+template <typename S, typename D> __device__ __forceinline__ S mul_sd(S a, D b) { return a * S(b); }
+template <> __device__ __forceinline__ dsf mul_sd<dsf, float>(dsf a, float b) { return ds_mul(a, b); }
+template <typename S, typename D> __device__ __forceinline__ S mul_dd(D a, D b) { return S(a) * S(b); }
+template <> __device__ __forceinline__ dsf mul_dd<dsf, float>(float a, float b) { return ds_mul(a, b); }
+// Re(conj(a) b)
+template <typename S, typename CS, typename CD> __device__ __forceinline__ S dot_sd(CS a, CD b) {
+  return mul_sd<S>(a.x, b.x) + mul_sd<S>(a.y, b.y);
+}
 
 // s1 = sum k |v|^2, s2 = sum k^2 |v|^2 over this thread's modes (k = xi[t + q Tl]):
 // Parseval's sums of the rotation and (twice) the kinetic symbol.
@@ -736,8 +761,8 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
 #pragma unroll
       for (int q = 0; q < E; ++q) {
         if (retract) {
-          const CS d = cconv<TS>(pq[q]);
-          ph[q] = cmk<CS>(cc * ph[q].x + ss * d.x, cc * ph[q].y + ss * d.y);
+          const CD d = pq[q];
+          ph[q] = cmk<CS>(cc * ph[q].x + mul_sd<TS>(ss, d.x), cc * ph[q].y + mul_sd<TS>(ss, d.y));
           phi_out[base + t + q * Tl] = ph[q];
         }
         v[q] = cconv<TF>(ph[q]);
@@ -785,7 +810,8 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
     const TS lam = num_as<TS>(S.lam);
     const TS alpha = num_as<TS>(S.alpha);
     const TS eta = num_as<TS>(a.eta_n);
-    TS rmax = 0, r2 = 0, bad = 0;
+    TS rmax = 0, r2 = 0;
+    float bad = 0.0f;
     const int pre = pc_pre(S.pc);
     const bool uses_pv = pre != 0 || pc_post(S.pc) != 0;
 #pragma unroll
@@ -795,7 +821,7 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
       CS r = rin[g];
       if (a.solver) r = cmk<CS>(r.x - lam * ph.x, r.y - lam * ph.y);
       const TS den = alpha + V[g] + eta * (ph.x * ph.x + ph.y * ph.y);
-      bad += (den > TS(0) || !uses_pv) ? TS(0) : TS(1);
+      bad += (den > TS(0) || !uses_pv) ? 0.0f : 1.0f;
       const TS a2 = r.x * r.x + r.y * r.y;
       rmax = fmax(rmax, a2); r2 += a2;
       v[q] = cconv<TF>(cscale(r, pv_factor(den, pre)));
@@ -859,14 +885,13 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
       const TS den = alpha + vv[q] + eta * (ph[q].x * ph[q].x + ph[q].y * ph[q].y);
       const CD Prd = cconv<TD>(cscale(cconv<TS>(v[q]), pv_factor(den, post)));
       sbuf[g] = Prd;
-      const CS Pr = cconv<TS>(Prd);  // the stored direction, as later passes see it
+      // the moments take the stored direction, as later passes see it
       const CS r = cmk<CS>(hq[q].x - lam * ph[q].x, hq[q].y - lam * ph[q].y);
-      const CS pq = cconv<TS>(pp[q]);
-      a0 += r.x * Pr.x + r.y * Pr.y;
-      a1 += (r.x - ro[q].x) * Pr.x + (r.y - ro[q].y) * Pr.y;
-      a2 += Pr.x * ph[q].x + Pr.y * ph[q].y;
-      a3 += pq.x * ph[q].x + pq.y * ph[q].y;
-      a4 += r.x * pq.x + r.y * pq.y;
+      a0 += dot_sd<TS>(r, Prd);
+      a1 += dot_sd<TS>(cmk<CS>(r.x - ro[q].x, r.y - ro[q].y), Prd);
+      a2 += dot_sd<TS>(ph[q], Prd);
+      a3 += dot_sd<TS>(ph[q], pp[q]);
+      a4 += dot_sd<TS>(r, pp[q]);
       a5 += r.x * ph[q].x + r.y * ph[q].y;
       rprev[g] = r;
     }
@@ -885,14 +910,15 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
     for (int q = 0; q < E; ++q) {
       const long long g = base + t + q * Tl;
       const CS ph = phi[g], h = Hphi[g];
-      const CS pr = cconv<TS>(Pr[g]), pp = cconv<TS>(pbuf[g]);
-      const CD pnd = cconv<TD>(cmk<CS>(-pr.x + beta * pp.x - gamma * ph.x, -pr.y + beta * pp.y - gamma * ph.y));
-      const CS pn = cconv<TS>(pnd);  // moments of the stored p
+      const CS pr = cconv<TS>(Pr[g]);
+      const CD pp = pbuf[g];
+      const CD pnd = cconv<TD>(cmk<CS>(-pr.x + mul_sd<TS>(beta, pp.x) - gamma * ph.x,
+                                       -pr.y + mul_sd<TS>(beta, pp.y) - gamma * ph.y));
       v[q] = cconv<TF>(pnd);
       const TS u = ph.x * ph.x + ph.y * ph.y;
-      const TS vr = ph.x * pn.x + ph.y * pn.y;
-      const TS wq = pn.x * pn.x + pn.y * pn.y;
-      aR += h.x * pn.x + h.y * pn.y;
+      const TS vr = dot_sd<TS>(ph, pnd);  // moments of the stored p
+      const TS wq = mul_dd<TS>(pnd.x, pnd.x) + mul_dd<TS>(pnd.y, pnd.y);
+      aR += dot_sd<TS>(h, pnd);
       aV += V[g] * wq;
       aW1 += wq; aUV += u * vr; aV2 += vr * vr; aUW += u * wq; aVW += vr * wq; aW2 += wq * wq; aRho += vr;
     }
