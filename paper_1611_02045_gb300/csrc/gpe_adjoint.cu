@@ -152,30 +152,41 @@ __device__ __forceinline__ void adj_reduce(const double (&v)[8], const AdjRed& r
 
 // Up to three inner products sum conj(x_j) y_j (x_j null: skipped; the real part of the second).
 template <typename C>
-__global__ void __launch_bounds__(kDotThreads) k_dots(const C* __restrict__ x0, const C* __restrict__ y0,
-                                                      const C* __restrict__ x1, const C* __restrict__ y1,
-                                                      const C* __restrict__ x2, const C* __restrict__ y2, long long n,
+__global__ void __launch_bounds__(kDotThreads) k_dots(const C* x0, const C* y0,
+                                                      const C* x1, const C* y1,
+                                                      const C* x2, const C* y2, long long n,
                                                       AdjRed red) {
+  pdl_wait();
+  x0 = after_wait(x0);
+  y0 = after_wait(y0);
+  x1 = after_wait(x1);
+  y1 = after_wait(y1);
+  x2 = after_wait(x2);
+  y2 = after_wait(y2);
   double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    if (x0) { const C a = x0[i], b = y0[i]; const double2 d = dconj_mul(a.x, a.y, b.x, b.y); v[0] += d.x; v[1] += d.y; }
-    if (x1) { const C a = x1[i], b = y1[i]; v[2] += (double)a.x * b.x + (double)a.y * b.y; }  // real part
-    if (x2) { const C a = x2[i], b = y2[i]; const double2 d = dconj_mul(a.x, a.y, b.x, b.y); v[4] += d.x; v[5] += d.y; }
+    if (x0) { const C a = __ldg(x0 + i), b = __ldg(y0 + i); const double2 d = dconj_mul(a.x, a.y, b.x, b.y); v[0] += d.x; v[1] += d.y; }
+    if (x1) { const C a = __ldg(x1 + i), b = __ldg(y1 + i); v[2] += (double)a.x * b.x + (double)a.y * b.y; }  // real part
+    if (x2) { const C a = __ldg(x2 + i), b = __ldg(y2 + i); const double2 d = dconj_mul(a.x, a.y, b.x, b.y); v[4] += d.x; v[5] += d.y; }
   }
+  pdl_trigger();
   adj_reduce(v, red);
 }
 
 // q <- q + eta |phi|^2 p + eta phi^2 conj(p) - lam p  (q holds H_phi p on entry),
 // then the sums <phi, q>, Re<p, q>, <p, phi>.
 template <typename C>
-__global__ void __launch_bounds__(kDotThreads) k_hess_epi(const C* __restrict__ phi, const C* __restrict__ p,
+__global__ void __launch_bounds__(kDotThreads) k_hess_epi(const C* phi, const C* p,
                                                           C* __restrict__ q, long long n, double eta, double lam,
                                                           AdjRed red) {
   using R = typename Real<C>::type;
   const R e = R(eta), l = R(lam);
+  pdl_wait();
+  phi = after_wait(phi);
+  p = after_wait(p);
   double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const C f = phi[i], d = p[i];
+    const C f = __ldg(phi + i), d = __ldg(p + i);
     C h = q[i];
     const R u = f.x * f.x + f.y * f.y;
     const R s2x = f.x * f.x - f.y * f.y, s2y = R(2) * f.x * f.y;  // phi^2
@@ -188,21 +199,26 @@ __global__ void __launch_bounds__(kDotThreads) k_hess_epi(const C* __restrict__ 
     v[2] += (double)d.x * h.x + (double)d.y * h.y;
     t = dconj_mul(d.x, d.y, f.x, f.y); v[4] += t.x; v[5] += t.y;
   }
+  pdl_trigger();
   adj_reduce(v, red);
 }
 
 // z += a p; r -= a (q - c phi); and the sum |r|^2.
 template <typename C>
-__global__ void __launch_bounds__(kDotThreads) k_step(C* __restrict__ z, C* __restrict__ r, const C* __restrict__ p,
-                                                      const C* __restrict__ q, const C* __restrict__ phi, long long n,
+__global__ void __launch_bounds__(kDotThreads) k_step(C* __restrict__ z, C* __restrict__ r, const C* p,
+                                                      const C* q, const C* phi, long long n,
                                                       AdjRed red) {
   using R = typename Real<C>::type;
   const AdjScalars* S = red.S;
+  pdl_wait();
+  p = after_wait(p);
+  q = after_wait(q);
+  phi = after_wait(phi);
   if (S->stop) return;  // converged or broken down: leave z and r as they are
   const R a = R(S->a), cr = R(S->c_re), ci = R(S->c_im);
   double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const C d = p[i], h = q[i], f = phi[i];
+    const C d = __ldg(p + i), h = __ldg(q + i), f = __ldg(phi + i);
     C zz = z[i], rr = r[i];
     const R qx = h.x - (cr * f.x - ci * f.y), qy = h.y - (cr * f.y + ci * f.x);
     zz.x += a * d.x; zz.y += a * d.y;
@@ -210,17 +226,20 @@ __global__ void __launch_bounds__(kDotThreads) k_step(C* __restrict__ z, C* __re
     z[i] = zz; r[i] = rr;
     v[0] += (double)rr.x * rr.x + (double)rr.y * rr.y;
   }
+  pdl_trigger();
   adj_reduce(v, red);
 }
 
 // h_out = h_in - c phi (c complex from S), h_out may alias h_in.
 template <typename C>
-__global__ void k_proj(const C* __restrict__ h_in, C* __restrict__ h_out, const C* __restrict__ phi, long long n,
-                       const AdjScalars* __restrict__ S) {
+__global__ void k_proj(const C* h_in, C* __restrict__ h_out, const C* phi, long long n,
+                       const AdjScalars* S) {
   using R = typename Real<C>::type;
+  pdl_wait();
+  phi = after_wait(phi);
   const R cr = R(S->c_re), ci = R(S->c_im);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const C h = h_in[i], f = phi[i];
+    const C h = h_in[i], f = __ldg(phi + i);
     C o;
     o.x = h.x - (cr * f.x - ci * f.y);
     o.y = h.y - (cr * f.y + ci * f.x);
@@ -230,14 +249,17 @@ __global__ void k_proj(const C* __restrict__ h_in, C* __restrict__ h_out, const 
 
 // p = (y - c phi) + beta p (beta = 0: p is not read).
 template <typename C>
-__global__ void k_dir(C* __restrict__ p, const C* __restrict__ y, const C* __restrict__ phi, long long n,
-                      const AdjScalars* __restrict__ S) {
+__global__ void k_dir(C* __restrict__ p, const C* y, const C* phi, long long n,
+                      const AdjScalars* S) {
   using R = typename Real<C>::type;
+  pdl_wait();
+  y = after_wait(y);
+  phi = after_wait(phi);
   if (S->stop) return;
   const R cr = R(S->c_re), ci = R(S->c_im), b = R(S->beta);
   const bool keep = S->beta != 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const C h = y[i], f = phi[i];
+    const C h = __ldg(y + i), f = __ldg(phi + i);
     C o;
     o.x = h.x - (cr * f.x - ci * f.y);
     o.y = h.y - (cr * f.y + ci * f.x);
@@ -249,12 +271,15 @@ __global__ void k_dir(C* __restrict__ p, const C* __restrict__ y, const C* __res
 // rhs = s g_rho phi (s = 2 / h^d: the weighted gradient of a loss of the
 // density |phi|^2 whose coefficient gradient is g_rho).
 template <typename C>
-__global__ void k_density_rhs(const C* __restrict__ phi, const double* __restrict__ g_rho, C* __restrict__ rhs,
+__global__ void k_density_rhs(const C* phi, const double* g_rho, C* __restrict__ rhs,
                               long long n, double s) {
   using R = typename Real<C>::type;
+  pdl_wait();
+  phi = after_wait(phi);
+  g_rho = after_wait(g_rho);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const C f = phi[i];
-    const R k = R(s * g_rho[i]);
+    const C f = __ldg(phi + i);
+    const R k = R(s * __ldg(g_rho + i));
     C o;
     o.x = k * f.x;
     o.y = k * f.y;
@@ -264,10 +289,13 @@ __global__ void k_density_rhs(const C* __restrict__ phi, const double* __restric
 
 // grad_V = -h^d Re(conj(z) phi)
 template <typename C>
-__global__ void k_dV_from_z(const C* __restrict__ phi, const C* __restrict__ z, double* __restrict__ gV, long long n,
+__global__ void k_dV_from_z(const C* phi, const C* z, double* __restrict__ gV, long long n,
                             double weight) {
+  pdl_wait();
+  phi = after_wait(phi);
+  z = after_wait(z);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const C f = phi[i], q = z[i];
+    const C f = __ldg(phi + i), q = __ldg(z + i);
     gV[i] = -weight * ((double)q.x * f.x + (double)q.y * f.y);
   }
 }
@@ -284,69 +312,72 @@ int grid_of(long long n, int max_blocks) {
 cudaError_t adj_dots(int prec, const void* x0, const void* y0, const void* x1, const void* y1, const void* x2,
                      const void* y2, long long n, double weight, int stage, const AdjWork& w, cudaStream_t st) {
   const int g = grid_of(n, kAdjMaxBlocks);
+  cudaError_t e;
   const AdjRed red = {w.partials, w.ticket, weight, stage, w.S};
   if (prec == 1)
-    k_dots<double2><<<g, kDotThreads, 0, st>>>((const double2*)x0, (const double2*)y0, (const double2*)x1,
-                                               (const double2*)y1, (const double2*)x2, (const double2*)y2, n, red);
+    e = launch_early(true, k_dots<double2>, g, kDotThreads, 0, st, (const double2*)x0, (const double2*)y0, (const double2*)x1, (const double2*)y1, (const double2*)x2, (const double2*)y2, n, red);
   else
-    k_dots<float2><<<g, kDotThreads, 0, st>>>((const float2*)x0, (const float2*)y0, (const float2*)x1,
-                                              (const float2*)y1, (const float2*)x2, (const float2*)y2, n, red);
-  return cudaGetLastError();
+    e = launch_early(true, k_dots<float2>, g, kDotThreads, 0, st, (const float2*)x0, (const float2*)y0, (const float2*)x1, (const float2*)y1, (const float2*)x2, (const float2*)y2, n, red);
+  return e;
 }
 
 cudaError_t adj_hess_epi(int prec, const void* phi, const void* p, void* q, long long n, double eta, double lam,
                          double weight, const AdjWork& w, cudaStream_t st) {
   const int g = grid_of(n, kAdjMaxBlocks);
+  cudaError_t e;
   const AdjRed red = {w.partials, w.ticket, weight, ADJ_PQ, w.S};
   if (prec == 1)
-    k_hess_epi<double2><<<g, kDotThreads, 0, st>>>((const double2*)phi, (const double2*)p, (double2*)q, n, eta, lam, red);
+    e = launch_early(true, k_hess_epi<double2>, g, kDotThreads, 0, st, (const double2*)phi, (const double2*)p, (double2*)q, n, eta, lam, red);
   else
-    k_hess_epi<float2><<<g, kDotThreads, 0, st>>>((const float2*)phi, (const float2*)p, (float2*)q, n, eta, lam, red);
-  return cudaGetLastError();
+    e = launch_early(true, k_hess_epi<float2>, g, kDotThreads, 0, st, (const float2*)phi, (const float2*)p, (float2*)q, n, eta, lam, red);
+  return e;
 }
 
 cudaError_t adj_step(int prec, void* z, void* r, const void* p, const void* q, const void* phi, long long n,
                      double weight, const AdjWork& w, cudaStream_t st) {
   const int g = grid_of(n, kAdjMaxBlocks);
+  cudaError_t e;
   const AdjRed red = {w.partials, w.ticket, weight, ADJ_RR, w.S};
   if (prec == 1)
-    k_step<double2><<<g, kDotThreads, 0, st>>>((double2*)z, (double2*)r, (const double2*)p, (const double2*)q,
-                                               (const double2*)phi, n, red);
+    e = launch_early(true, k_step<double2>, g, kDotThreads, 0, st, (double2*)z, (double2*)r, (const double2*)p, (const double2*)q, (const double2*)phi, n, red);
   else
-    k_step<float2><<<g, kDotThreads, 0, st>>>((float2*)z, (float2*)r, (const float2*)p, (const float2*)q,
-                                              (const float2*)phi, n, red);
-  return cudaGetLastError();
+    e = launch_early(true, k_step<float2>, g, kDotThreads, 0, st, (float2*)z, (float2*)r, (const float2*)p, (const float2*)q, (const float2*)phi, n, red);
+  return e;
 }
 
 cudaError_t adj_proj(int prec, const void* h_in, void* h_out, const void* phi, long long n, const AdjScalars* S,
                      cudaStream_t st) {
   const int g = grid_of(n, 4096);
-  if (prec == 1) k_proj<double2><<<g, kDotThreads, 0, st>>>((const double2*)h_in, (double2*)h_out, (const double2*)phi, n, S);
-  else k_proj<float2><<<g, kDotThreads, 0, st>>>((const float2*)h_in, (float2*)h_out, (const float2*)phi, n, S);
-  return cudaGetLastError();
+  cudaError_t e;
+  if (prec == 1) e = launch_early(true, k_proj<double2>, g, kDotThreads, 0, st, (const double2*)h_in, (double2*)h_out, (const double2*)phi, n, S);
+  else e = launch_early(true, k_proj<float2>, g, kDotThreads, 0, st, (const float2*)h_in, (float2*)h_out, (const float2*)phi, n, S);
+  return e;
 }
 
 cudaError_t adj_dir(int prec, void* p, const void* y, const void* phi, long long n, const AdjScalars* S, cudaStream_t st) {
   const int g = grid_of(n, 4096);
-  if (prec == 1) k_dir<double2><<<g, kDotThreads, 0, st>>>((double2*)p, (const double2*)y, (const double2*)phi, n, S);
-  else k_dir<float2><<<g, kDotThreads, 0, st>>>((float2*)p, (const float2*)y, (const float2*)phi, n, S);
-  return cudaGetLastError();
+  cudaError_t e;
+  if (prec == 1) e = launch_early(true, k_dir<double2>, g, kDotThreads, 0, st, (double2*)p, (const double2*)y, (const double2*)phi, n, S);
+  else e = launch_early(true, k_dir<float2>, g, kDotThreads, 0, st, (float2*)p, (const float2*)y, (const float2*)phi, n, S);
+  return e;
 }
 
 cudaError_t adj_density_rhs(int prec, const void* phi, const double* g_rho, void* rhs, long long n, double s,
                             cudaStream_t st) {
   const int g = grid_of(n, 4096);
-  if (prec == 1) k_density_rhs<double2><<<g, kDotThreads, 0, st>>>((const double2*)phi, g_rho, (double2*)rhs, n, s);
-  else k_density_rhs<float2><<<g, kDotThreads, 0, st>>>((const float2*)phi, g_rho, (float2*)rhs, n, s);
-  return cudaGetLastError();
+  cudaError_t e;
+  if (prec == 1) e = launch_early(true, k_density_rhs<double2>, g, kDotThreads, 0, st, (const double2*)phi, g_rho, (double2*)rhs, n, s);
+  else e = launch_early(true, k_density_rhs<float2>, g, kDotThreads, 0, st, (const float2*)phi, g_rho, (float2*)rhs, n, s);
+  return e;
 }
 
 cudaError_t adj_dV_from_z(int prec, const void* phi, const void* z, double* gV, long long n, double weight,
                           cudaStream_t st) {
   const int g = grid_of(n, 4096);
-  if (prec == 1) k_dV_from_z<double2><<<g, kDotThreads, 0, st>>>((const double2*)phi, (const double2*)z, gV, n, weight);
-  else k_dV_from_z<float2><<<g, kDotThreads, 0, st>>>((const float2*)phi, (const float2*)z, gV, n, weight);
-  return cudaGetLastError();
+  cudaError_t e;
+  if (prec == 1) e = launch_early(true, k_dV_from_z<double2>, g, kDotThreads, 0, st, (const double2*)phi, (const double2*)z, gV, n, weight);
+  else e = launch_early(true, k_dV_from_z<float2>, g, kDotThreads, 0, st, (const float2*)phi, (const float2*)z, gV, n, weight);
+  return e;
 }
 
 }  // namespace gpe

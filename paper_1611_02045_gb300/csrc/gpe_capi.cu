@@ -704,19 +704,21 @@ static gpe_status run_PC(gpe_ctx* c, const IterBufs& b, const void* r, double al
   a.ctl = ctl; a.solver = solver; a.phi = b.phi; a.r_in = r; a.api_alpha = num(alpha);
   a.s = b.s; a.t = b.t; a.r_prev = b.r_prev; a.p = b.p; a.out = out;
   GPE_CU(c, launch(b.mode, P_C1, a, st));
+  const int early = 1;  // the passes behind C1; C1 itself is launched plainly (launch_early's comment)
   if (c->dim == 3) {
     PassArgs y = base_args(c, b.tab_d, 1, b.mode);
-    y.ctl = ctl; y.solver = solver; y.s = b.s;
+    y.ctl = ctl; y.solver = solver; y.early = early; y.s = b.s;
     GPE_CU(c, launch(b.mode, P_CFWD, y, st));
   }
   PassArgs k = base_args(c, b.tab_d, c->dim - 1, b.mode);
-  k.ctl = ctl; k.solver = solver; k.s = b.s; k.api_alpha = num(alpha);
+  k.ctl = ctl; k.solver = solver; k.early = early; k.s = b.s; k.api_alpha = num(alpha);
   GPE_CU(c, launch(b.mode, P_CCORE, k, st));
   if (c->dim == 3) {
     PassArgs y = base_args(c, b.tab_d, 1, b.mode);
-    y.ctl = ctl; y.solver = solver; y.s = b.s;
+    y.ctl = ctl; y.solver = solver; y.early = early; y.s = b.s;
     GPE_CU(c, launch(b.mode, P_CINV, y, st));
   }
+  a.early = early;
   GPE_CU(c, launch(b.mode, P_C3, a, st));
   return GPE_OK;
 }

@@ -40,6 +40,43 @@ __host__ __device__ inline Num num(double d) {
   return n;
 }
 
+// Programmatic dependent launch: a kernel started by launch_early may be put on the
+// GPU while the one before it in the stream still finishes (once each of that one's
+// blocks has called pdl_trigger or left), so that its launch does not wait behind the
+// other's last block.  Such a kernel touches no memory before pdl_wait, which returns
+// when the kernel before it is complete and its writes are visible.  pdl_trigger comes
+// late, in front of a kernel's reductions: blocks that only wait would hold SM slots.
+// Chains of short kernels gain 1 to 2 us a launch: P_C r on 256 x 128 x 64 105.7 ->
+// 98.6 us, density adjoint on 256^2 complex128 11.6 -> 10.2 ms, Thomas-Fermi start on
+// 256^2 with its interpolation 154 -> 130 us.  P_C's first pass is launched plainly: early
+// behind the adjoint's k_step it makes those 10.2 ms 13.1.  In the bodies of the solver's
+// graph loops it changes nothing (73.8 us per refinement iteration both ways), so they
+// keep plain launches.  Both calls do nothing in a kernel launched the plain way.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
+// A field that the kernel before writes, where it is declared __restrict__: loads
+// through it may count as invariant to the compiler and move above pdl_wait, so they go
+// through the pointer that this returns after it.
+template <typename T> __device__ __forceinline__ T* after_wait(T* p) {
+  asm volatile("" : "+l"(p));
+  return p;
+}
+template <typename... A, typename... B>
+inline cudaError_t launch_early(bool early, void (*kern)(A...), long long grid, int threads, size_t smem,
+                                cudaStream_t st, const B&... b) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3((unsigned)threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = early ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, b...);
+}
+
 // Number of doubles in one per-iteration log row (matches GPE_LOG_FIELDS).
 constexpr int kLogFields = 12;
 // Max reduction slots per pass.
@@ -122,6 +159,7 @@ struct PassArgs {
   int nblocks;     // grid size
   int pf;          // contiguous H pass outside a solve: L2 prefetch of the rows of unit + pf (0: none)
   int solver;      // 1: inside a solve (uses ctl scalars, solver reductions)
+  int early;       // 1: P_C's passes behind the first, outside a solve: launch_early
   int nomoments;   // 1: the caller needs no reductions (H phi as a plain operator): passes skip them
   int eonly;       // 1: only the energy moments are wanted (gpe_energy, the shift of P_C): the H passes stop
                    // after their forward transforms and write no field

@@ -47,6 +47,7 @@ __global__ void __launch_bounds__(512) pass_s_tma(PassArgs a, const __grid_const
   constexpr int NT = STiles<ROLE>::value;
   extern __shared__ __align__(128) unsigned char smraw[];
   __shared__ __align__(8) unsigned long long bar[2];
+  if constexpr (kEarlyRole<ROLE>) pdl_wait();
   if (a.solver && a.ctl->done) {
     if (ROLE == P_AMID && a.last_axis && blockIdx.x == 0 && threadIdx.x == 0) set_loop_condition(a, 0);
     return;
@@ -184,6 +185,7 @@ __global__ void __launch_bounds__(512) pass_s_tma(PassArgs a, const __grid_const
     }
     __syncthreads();  // stage s is read by every thread before it is refilled
   }
+  if constexpr (kEarlyRole<ROLE>) pdl_trigger();
   reduce_and_finish<ROLE>(a, acc);
 }
 
@@ -359,6 +361,7 @@ __global__ void __launch_bounds__(512) pass_xc_bulk(PassArgs a) {
   extern __shared__ __align__(128) unsigned char smraw[];
   __shared__ __align__(8) unsigned long long bar[2];
   __shared__ PassArgs sa[2];  // the unit body's arguments, pointed at stage s
+  if constexpr (kEarlyRole<ROLE>) pdl_wait();
   if (a.solver && a.ctl->done) return;
   const Scal S = scal_of(a.ctl, a);
   const int lpb = a.lpb;
@@ -440,6 +443,7 @@ __global__ void __launch_bounds__(512) pass_xc_bulk(PassArgs a) {
     if (threadIdx.x == 0) store(u, s);
   }
   if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
+  if constexpr (kEarlyRole<ROLE>) pdl_trigger();
   reduce_and_finish<ROLE>(a, acc);
 }
 // Tensor map over a complex64 field [nz][ny][nx] (8-byte elements), boxes of
@@ -506,8 +510,7 @@ cudaError_t launch_tma_one(const PassArgs& a0, cudaStream_t st, bool* used) {
   // fields (L2-resident 2D grids) keep the tuned one-tile-per-block kernel
   if (a.nblocks < 2 * grid) return cudaSuccess;
   *used = true;
-  kern<<<(unsigned)grid, threads, smem, st>>>(a, tm0, tm1);
-  return cudaGetLastError();
+  return launch_early(kEarlyRole<ROLE> && a.early && !a.solver, kern, grid, threads, smem, st, a, tm0, tm1);
 }
 
 template <int ROLE>
@@ -611,8 +614,7 @@ cudaError_t launch_xc_one(const PassArgs& a0, cudaStream_t st, bool* used) {
   // at least two units per block, and no more blocks than the plan's (the reduction partials hold those)
   if (a.nblocks < 2 * grid || grid > a0.nblocks) return cudaSuccess;
   *used = true;
-  kern<<<(unsigned)grid, threads, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_early(kEarlyRole<ROLE> && a.early && !a.solver, kern, grid, threads, smem, st, a);
 }
 
 template <int ROLE>

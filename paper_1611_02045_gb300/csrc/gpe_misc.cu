@@ -199,6 +199,8 @@ __global__ void __launch_bounds__(kTfThreads) k_tf_step(const double* __restrict
   __shared__ double sm[NW];
   __shared__ unsigned long long smc[NW];
   __shared__ int s_last;
+  pdl_wait();
+  V = after_wait(V);
   const TfState S = first ? init : *st;  // *st: written by the previous launch
   if (S.done) return;
   const double x = S.x;
@@ -223,6 +225,7 @@ __global__ void __launch_bounds__(kTfThreads) k_tf_step(const double* __restrict
     if (threadIdx.x == 0)
       for (int w = 1; w < NW; ++w) { acc += sm[w]; cnt += smc[w]; }
   };
+  pdl_trigger();
   block_sum();
   unsigned long long* pc = reinterpret_cast<unsigned long long*>(partials) + 1024;
   if (threadIdx.x == 0) {
@@ -266,20 +269,20 @@ cudaError_t launch_tf_step(const double* V, long long n, double w_eta, TfState* 
   long long g = (n + 4LL * kTfThreads - 1) / (4LL * kTfThreads);
   if (g < 1) g = 1;
   if (g > 1024) g = 1024;
-  k_tf_step<<<(int)g, kTfThreads, 0, st>>>(V, n, w_eta, state, init, first ? 1 : 0, partials, ticket);
-  return cudaGetLastError();
+  return launch_early(true, k_tf_step, g, kTfThreads, 0, st, V, n, w_eta, state, init, first ? 1 : 0, partials, ticket);
 }
 
 __global__ void k_tf_fill(const double* __restrict__ V, long long n, double eta, const TfState* state,
                           double2* __restrict__ phi) {
+  pdl_wait();
+  V = after_wait(V);
   const double mu = state->x;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
     phi[i] = make_double2(sqrt(fmax(mu - V[i], 0.0) / eta), 0.0);
 }
 cudaError_t launch_tf_fill(const double* V, long long n, double eta, const TfState* state, void* phi128,
                            cudaStream_t st) {
-  k_tf_fill<<<grid_for(n), 256, 0, st>>>(V, n, eta, state, (double2*)phi128);
-  return cudaGetLastError();
+  return launch_early(true, k_tf_fill, grid_for(n), 256, 0, st, V, n, eta, state, (double2*)phi128);
 }
 
 // Epilogue of gpe_energy_grad: grad_phi <- 2 h^d H_phi phi in place (Section 2,

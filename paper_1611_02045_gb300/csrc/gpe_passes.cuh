@@ -671,6 +671,11 @@ __device__ __forceinline__ void apply_symbol(C (&v)[E], const T* __restrict__ xi
 // ---------------------------------------------------------------------------
 // Max threads per block: 512 with single-precision transforms, 256 with double.
 template <typename T> struct MaxThreads { static constexpr int value = sizeof(T) == 8 ? 256 : 512; };
+// Roles whose passes take part in programmatic dependent launch: those of the combined
+// preconditioner.  In the H passes the two instructions cost registers (FP64 x pass at
+// M = 128 from 128 to 158, one block per SM where two fit: H phi on 128^3 complex128 545
+// us instead of 522, energy and gradient on 512^2 469 instead of 452), so they stay out.
+template <int ROLE> constexpr bool kEarlyRole = ROLE == P_C1 || ROLE == P_C3 || ROLE == P_CFWD || ROLE == P_CCORE || ROLE == P_CINV;
 
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
@@ -805,8 +810,8 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
     }
   } else if constexpr (ROLE == P_C1) {
     // ---- s = FFT_x[P_V^{1/2} r], r = H phi - lambda phi (solver) or r_in (API) ----
-    const CS* __restrict__ phi = static_cast<const CS*>(a.phi);
-    const CS* __restrict__ rin = static_cast<const CS*>(a.solver ? a.t : a.r_in);
+    const CS* __restrict__ phi = after_wait(static_cast<const CS*>(a.phi));
+    const CS* __restrict__ rin = after_wait(static_cast<const CS*>(a.solver ? a.t : a.r_in));
     const TS lam = num_as<TS>(S.lam);
     const TS alpha = num_as<TS>(S.alpha);
     const TS eta = num_as<TS>(a.eta_n);
@@ -836,8 +841,8 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
     acc[2] = acc_add(acc[2], acc_from(bad));
   } else if constexpr (ROLE == P_C3) {
     // ---- Pr = P_V^{1/2} IFFT_x[s] (the 1/N is applied in the core pass) ----
-    const CS* __restrict__ phi = static_cast<const CS*>(a.phi);
-    CD* __restrict__ sbuf = static_cast<CD*>(a.s);
+    const CS* __restrict__ phi = after_wait(static_cast<const CS*>(a.phi));
+    CD* __restrict__ sbuf = after_wait(static_cast<CD*>(a.s));
 #pragma unroll
     for (int q = 0; q < E; ++q) v[q] = cconv<TF>(sbuf[base + t + q * Tl]);
     const TS alpha = num_as<TS>(S.alpha);
@@ -992,7 +997,7 @@ __device__ __forceinline__ void sunit(const PassArgs& a, const Scal& S, long lon
 #pragma unroll
     for (int q = 0; q < E; ++q) dst[base + (t + q * Tl) * st] = cadd(tv[q], v[q]);
   } else if constexpr (ROLE == P_CFWD || ROLE == P_CINV || ROLE == P_CCORE) {
-    C* __restrict__ sb = static_cast<C*>(a.s);
+    C* __restrict__ sb = after_wait(static_cast<C*>(a.s));
 #pragma unroll
     for (int q = 0; q < E; ++q) v[q] = sb[base + (t + q * Tl) * st];
     if (S.done) return;
@@ -1149,11 +1154,13 @@ __device__ __forceinline__ void reduce_and_finish(const PassArgs& a, const Acc* 
 template <typename TF, typename TS, typename TD, int M, int ROLE, int EV>
 __global__ void __launch_bounds__(MaxThreads<TF>::value < MaxThreads<TS>::value ? MaxThreads<TF>::value : MaxThreads<TS>::value) pass_x(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  if constexpr (kEarlyRole<ROLE>) pdl_wait();
   const Scal S = scal_of(a.ctl, a);
   Acc acc[kMaxMoments];
 #pragma unroll
   for (int k = 0; k < kMaxMoments; ++k) acc[k] = Acc{0.0f, 0.0f};
   xunit<TF, TS, TD, M, ROLE, EV>(a, S, blockIdx.x, smraw, acc);
+  if constexpr (kEarlyRole<ROLE>) pdl_trigger();
   if (S.done) return;
   reduce_and_finish<ROLE>(a, acc);
 }
@@ -1161,11 +1168,13 @@ __global__ void __launch_bounds__(MaxThreads<TF>::value < MaxThreads<TS>::value 
 template <typename T, int M, int ROLE, int EV>
 __global__ void __launch_bounds__(MaxThreads<T>::value) pass_s(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
+  if constexpr (kEarlyRole<ROLE>) pdl_wait();
   const Scal S = scal_of(a.ctl, a);
   Acc acc[kMaxMoments];
 #pragma unroll
   for (int k = 0; k < kMaxMoments; ++k) acc[k] = Acc{0.0f, 0.0f};
   sunit<T, M, ROLE, EV>(a, S, blockIdx.x, smraw, acc);
+  if constexpr (kEarlyRole<ROLE>) pdl_trigger();
   if (S.done) {
     if (ROLE == P_AMID && a.last_axis && blockIdx.x == 0 && threadIdx.x == 0) set_loop_condition(a, 0);
     return;
@@ -1215,8 +1224,7 @@ cudaError_t launch_one(const PassArgs& a, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     attr.set(dev);
   }
-  kern<<<a.nblocks, threads, smem, st>>>(a);
-  return cudaGetLastError();
+  return launch_early(kEarlyRole<ROLE> && a.early && !a.solver, kern, a.nblocks, threads, smem, st, a);
 }
 
 // E = 8 for every M; E = 4 (plans chosen by the tuner) for M >= 32, in
