@@ -81,6 +81,8 @@ struct gpe_ctx {
   int hbatch_rows = 16;  // rows per CTA of its streaming form (plan mode 3 width: 16 or 32)
   int* hflow_ctr = nullptr;  // counters of gpe_apply_H_batch's dataflow form (zero between launches)
   int hflow_cap = 0;
+  int* hflow_old[24] = {};  // outgrown counters (sizes at least double): a graph captured with them may still run
+  int hflow_nold = 0;
   int hbatch_E = 8;      // values per thread of gpe_apply_H_batch's cluster kernel (plan mode 3):
                          // 16 (streaming form) by default in single precision for n >= 64
   Pinned* pinned = nullptr;
@@ -307,6 +309,7 @@ static void free_ctx(gpe_ctx* c) {
   if (c->pinned) cudaFreeHost(c->pinned);
   cudaFree(c->adj_s); cudaFree(c->adj_partials);
   cudaFree(c->hflow_ctr);
+  for (int* p : c->hflow_old) cudaFree(p);  // (null: nothing)
   cudaFree(c->ctl_solve); cudaFree(c->ctl_api); cudaFree(c->partials); cudaFree(c->ticket); cudaFree(c->log_dev);
   if (c->cap) cudaStreamDestroy(c->cap);
   delete c;
@@ -455,10 +458,11 @@ static gpe_status try_flow(gpe_ctx* c, int nplanes, long long vstride, const voi
     GPE_CU(c, cudaStreamIsCapturing(c->st, &cs));
     if (cs != cudaStreamCaptureStatusNone) return GPE_OK;  // no allocation under capture: the other forms
     const size_t cap = need > 2 * (size_t)c->hflow_cap ? need : 2 * (size_t)c->hflow_cap;
-    if (c->hflow_ctr) GPE_CU(c, cudaFree(c->hflow_ctr));
-    c->hflow_ctr = nullptr;
+    int* ctr = nullptr;
+    GPE_CU(c, cudaMalloc(&ctr, cap * sizeof(int)));
+    if (c->hflow_ctr && c->hflow_nold < 24) c->hflow_old[c->hflow_nold++] = c->hflow_ctr;
+    c->hflow_ctr = ctr;
     c->hflow_cap = 0;
-    GPE_CU(c, cudaMalloc(&c->hflow_ctr, cap * sizeof(int)));
     GPE_CU(c, cudaMemsetAsync(c->hflow_ctr, 0, cap * sizeof(int), c->st));
     c->hflow_cap = (int)cap;
   }

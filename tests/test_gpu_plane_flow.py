@@ -128,3 +128,25 @@ def test_batch_larger_than_the_counters_under_capture(G):
         s.synchronize()
         assert close(out, ref)
         del graph
+
+
+def test_captured_batch_outlives_a_growth_of_the_counters(G):
+    """A batch captured with the context's first counters, replayed after a larger batch
+    has outgrown them: the same bits as before."""
+    M, nb, more = 64, 800, 1100
+    n, L = (M, M), (8.0, 8.0)
+    s = torch.cuda.Stream()
+    f = field((more, M, M), 10)
+    torch.cuda.synchronize()
+    with torch.cuda.stream(s), G.Context(n, L, 30.0, 0.4, I.harmonic(n, L), prec=G.GPE_MIXED) as ctx:
+        out, ref, big = torch.zeros_like(f[:nb]), torch.empty_like(f[:nb]), torch.empty_like(f)
+        ctx.apply_H_batch(nb, f[:nb], f[:nb], ref)
+        s.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=s):
+            ctx.apply_H_batch(nb, f[:nb], f[:nb], out)
+        ctx.apply_H_batch(more, f, f, big)
+        graph.replay()
+        s.synchronize()
+        assert torch.equal(out, ref) and torch.equal(big[:nb], ref)
+        del graph
