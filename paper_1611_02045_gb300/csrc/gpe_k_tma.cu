@@ -130,10 +130,10 @@ __global__ void __launch_bounds__(512) pass_s_tma(PassArgs a, const __grid_const
       line_dft<M, E, -1>(v, ex, si, t, tw);
       const T rx = (a.axis == 1) ? -tab<T>(a.xc[0])[ix] : T(0);  // rotation symbol -omega x mu (y); none for z
       if (!a.nomoments) {
-        T s1, s2;
-        symbol_sums<E>(v, xia, t, Tl, s1, s2);
-        acc[0] = acc_add(acc[0], acc_from(T(0.5) * s2 * invM));
-        acc[1] = acc_add(acc[1], acc_from(rx * s1 * invM));
+        T akin, arot;
+        symbol_sums<E>(v, xia, t, Tl, rx, akin, arot);
+        acc[0] = acc_add(acc[0], acc_from(akin * invM));
+        acc[1] = acc_add(acc[1], acc_from(arot * invM));
       }
       if (!a.eonly) {
         apply_symbol<E>(v, xia, t, Tl, T(0.5) * invM, om * rx * invM);
@@ -288,10 +288,10 @@ __global__ void __launch_bounds__(512) pass_hx_bulk(PassArgs a, int second) {
     line_dft<M, E, -1, W>(v, sm, si, t, tw);
     const T y = tab<T>(a.xc[1])[iy];
     if (!a.nomoments) {  // the rotation symbol without omega (applied in finalize_H)
-      T s1, s2;
-      symbol_sums<E>(v, xi, t, Tl, s1, s2);
-      acc[0] = acc_add(acc[0], acc_from(T(0.5) * s2 * invM));
-      acc[1] = acc_add(acc[1], acc_from(y * s1 * invM));
+      T akin, arot;
+      symbol_sums<E>(v, xi, t, Tl, y, akin, arot);
+      acc[0] = acc_add(acc[0], acc_from(akin * invM));
+      acc[1] = acc_add(acc[1], acc_from(arot * invM));
     }
     if (!a.eonly) {
       apply_symbol<E>(v, xi, t, Tl, T(0.5) * invM, om * y * invM);
