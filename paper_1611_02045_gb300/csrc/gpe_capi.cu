@@ -218,6 +218,29 @@ static IterBufs iter_bufs(gpe_ctx* c, int mode) {
   return b;
 }
 
+// e^{-2 pi i m / M} (M in [8, 512] a power of two) to the nearest double, from the angles
+// of the first octant; cos(2.0 * M_PI * m / M) carries the rounding of its angle, up to
+// 5.8 units of 2^-53.  The octant of M = 512 serves every M and is computed once per
+// process: extended precision is slow where it is emulated.
+static void unit_root(int m, int M, double* re, double* im) {
+  struct Octant {
+    double c[65], s[65];
+    Octant() {
+      for (int j = 0; j <= 64; ++j) {
+        const long double a = 3.14159265358979323846264338327950288L * j / 256;
+        c[j] = (double)std::cos(a);
+        s[j] = (double)std::sin(a);
+      }
+    }
+  };
+  static const Octant o;
+  const int i = m * (512 / M), r = i % 128;
+  const double c = r <= 64 ? o.c[r] : o.s[128 - r], s = r <= 64 ? o.s[r] : o.c[128 - r];
+  const double cs[4] = {c, -s, -c, s}, sn[4] = {s, c, -s, -c};  // turned by quarter turns
+  *re = cs[i / 128];
+  *im = -sn[i / 128];
+}
+
 template <typename T>
 static cudaError_t upload_tables(gpe_ctx* c, PrecBufs& b) {
   for (int i = 0; i < c->dim; ++i) {
@@ -228,8 +251,10 @@ static cudaError_t upload_tables(gpe_ctx* c, PrecBufs& b) {
       const int pp = p < M / 2 ? p : p - M;  // xi_p = p pi / L, p = -M/2 .. M/2-1
       xi[p] = (T)(pp * M_PI / L);
       xc[p] = (T)(-L + p * (2.0 * L / M));   // x_k = -L + k h
-      tw[2 * p] = (T)std::cos(2.0 * M_PI * p / M);
-      tw[2 * p + 1] = (T)(-std::sin(2.0 * M_PI * p / M));
+      double re, im;
+      unit_root(p, M, &re, &im);
+      tw[2 * p] = (T)re;
+      tw[2 * p + 1] = (T)im;
     }
     cudaError_t e;
     if ((e = cudaMalloc(&b.xi[i], M * sizeof(T))) != cudaSuccess) return e;

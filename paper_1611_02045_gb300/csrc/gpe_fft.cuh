@@ -17,6 +17,8 @@
 #pragma once
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "gpe_ds.cuh"
 
 namespace gpe {
@@ -109,13 +111,14 @@ template <int DIR, typename C> __device__ __forceinline__ void dft8(C (&x)[8]) {
   x[3] = cadd(e3, t3); x[7] = csub(e3, t3);
 }
 
-// FP64: the products with cos(pi/4) fused into the last level's sums
-template <int DIR> __device__ __forceinline__ void dft8(double2 (&x)[8]) {
+// FP64 radix 8 after its first level (x[r] = x_r + x_{r+4}, x[r + 4] = x_r - x_{r+4}, r < 4):
+// the products with cos(pi/4) are fused into the last level's sums, which takes four
+// instructions less than the form above and rounds less.
+template <int DIR> __device__ __forceinline__ void dft8_rest(double2 (&x)[8]) {
   const double h = 0.70710678118654752440;
-  double2 e0 = x[0], e1 = x[2], e2 = x[4], e3 = x[6];
-  double2 o0 = x[1], o1 = x[3], o2 = x[5], o3 = x[7];
-  dft4<DIR>(e0, e1, e2, e3);
-  dft4<DIR>(o0, o1, o2, o3);
+  const double2 d2 = cmul_i<DIR>(x[6]), d3 = cmul_i<DIR>(x[7]);
+  const double2 e0 = cadd(x[0], x[2]), e2 = csub(x[0], x[2]), e1 = cadd(x[4], d2), e3 = csub(x[4], d2);
+  const double2 o0 = cadd(x[1], x[3]), o2 = csub(x[1], x[3]), o1 = cadd(x[5], d3), o3 = csub(x[5], d3);
   const double2 s1 = DIR < 0 ? make_double2(o1.x + o1.y, o1.y - o1.x) : make_double2(o1.x - o1.y, o1.y + o1.x);
   const double2 t2 = cmul_i<DIR>(o2);
   const double2 s3 = DIR < 0 ? make_double2(o3.y - o3.x, -(o3.x + o3.y)) : make_double2(-(o3.x + o3.y), o3.x - o3.y);
@@ -125,6 +128,11 @@ template <int DIR> __device__ __forceinline__ void dft8(double2 (&x)[8]) {
   x[2] = cadd(e2, t2); x[6] = csub(e2, t2);
   x[3] = make_double2(fma(h, s3.x, e3.x), fma(h, s3.y, e3.y));
   x[7] = make_double2(fma(-h, s3.x, e3.x), fma(-h, s3.y, e3.y));
+}
+template <int DIR> __device__ __forceinline__ void dft8(double2 (&x)[8]) {
+#pragma unroll
+  for (int r = 0; r < 4; ++r) dft2<DIR>(x[r], x[r + 4]);
+  dft8_rest<DIR>(x);
 }
 
 template <int DIR, typename C> __device__ __forceinline__ void dft16(C (&x)[16]) {
@@ -164,78 +172,61 @@ template <int R, int DIR, typename C> __device__ __forceinline__ void dft_small(
 }
 
 // ---------------------------------------------------------------------------
-// Twiddled butterflies: (a, b) <- (a + W b, a - W b) with W = w (DIR = -1) or
-// conj(w) (DIR = +1); bfly_i: the same with W times -i (DIR = -1) or +i.  In
-// FP64, where every instruction holds the pipe, as six fused operations: two
-// per component of a + W b, and a - W b = 2 a - (a + W b) in one; product, sum
-// and difference apart take eight.
+// FP64 transforms with twiddles, y_m = sum_r (w^r x_r) e^{DIR 2 pi i r m / R} in place
+// (w^r taken in the sense of ctw), where every FP64 instruction holds the pipe: the
+// first level of radix-2 butterflies takes a = w^r x_r (r < R/2) and multiplies by
+// W = w^{r + R/2} in the sum itself, a + W b and a - W b as two fused operations per
+// component each, or (SHORT) a - W b as 2 a - (a + W b) in one, six operations in all
+// against eight, which carries the sum's rounding into the difference.
+//
+// Precision.  RMS error of a forward and inverse pair in units of the relative rounding,
+// emulated stage by stage with exact fused operations and twiddles to the nearest number:
+//    M, E     products, sums and   fused   SHORT   three levels of twiddled butterflies
+//             differences apart                    with w^4, w^2, w (cascaded)
+//    32, 8         1.703           1.680   1.711        1.888
+//    64, 8         1.923           1.872   1.905        2.152
+//   128, 8         2.127           2.065   2.128        2.356
+//   256, 8         2.251           2.200   2.253        2.546
+//   512, 8         2.459           2.381   2.440        2.718
+//   256, 4         2.230           2.217   2.307        2.581
+// SHORT is taken in radix 8, for E = 4 (whose passes are short of threads and gain an
+// eighth of their operations) and in a last radix 2 or 4 behind two radix-8 stages; in
+// M = 16 and 32 it would gain little.  The cascade takes as few operations with four
+// table entries instead of seven, and is 2% faster (H phi on 128^3 complex128 519 against
+// 531 us), but multiplies every value three times.  Measured, H f along one axis, error
+// in 2^-53 (twiddles from rounded angles and cascaded -> as it is): M = 128 2.56 -> 2.31
+// and (E = 4) 2.88 -> 2.25, M = 512 3.03 -> 2.79 and 3.39 -> 2.57; products apart and
+// rounded angles: 2.67, 2.52, 3.10, 3.04.
 // ---------------------------------------------------------------------------
-template <int DIR, typename C> __device__ __forceinline__ void bfly(C& a, C& b, C w) {
-  const C t = ctw<DIR>(b, w);
-  b = csub(a, t);
-  a = cadd(a, t);
-}
-template <int DIR, typename C> __device__ __forceinline__ void bfly_i(C& a, C& b, C w) {
-  const C t = cmul_i<DIR>(ctw<DIR>(b, w));
-  b = csub(a, t);
-  a = cadd(a, t);
-}
-template <int DIR> __device__ __forceinline__ void bfly(double2& a, double2& b, double2 w) {
+template <int DIR, bool SHORT> __device__ __forceinline__ void bfly(double2& a, double2& b, double2 w) {
   const double wi = DIR < 0 ? w.y : -w.y;
   const double2 y = make_double2(fma(-b.y, wi, fma(b.x, w.x, a.x)), fma(b.x, wi, fma(b.y, w.x, a.y)));
-  b = make_double2(fma(2.0, a.x, -y.x), fma(2.0, a.y, -y.y));
-  a = y;
-}
-template <int DIR> __device__ __forceinline__ void bfly_i(double2& a, double2& b, double2 w) {
-  // W b times -i (+i): (p, q) -> (q, -p) ((-q, p))
-  const double wi = DIR < 0 ? w.y : -w.y, sg = DIR < 0 ? 1.0 : -1.0;
-  const double2 y = make_double2(fma(sg * b.x, wi, fma(sg * b.y, w.x, a.x)),
-                                 fma(sg * b.y, wi, fma(-sg * b.x, w.x, a.y)));
-  b = make_double2(fma(2.0, a.x, -y.x), fma(2.0, a.y, -y.y));
+  if constexpr (SHORT)
+    b = make_double2(fma(2.0, a.x, -y.x), fma(2.0, a.y, -y.y));
+  else
+    b = make_double2(fma(b.y, wi, fma(-b.x, w.x, a.x)), fma(-b.x, wi, fma(-b.y, w.x, a.y)));
   a = y;
 }
 
-// y_m = sum_r (w^r x_r) e^{DIR 2 pi i r m / R} in place, w^r taken in the sense of
-// ctw: radix 2^k as k levels of twiddled radix-2 butterflies with twiddles
-// w^{R/2}, w^{R/4}, ... (times the level's roots of unity), so that R = 8 reads
-// four table entries instead of seven.  tw: e^{-2 pi i m / M} table, i: index of w.
-template <int R, int DIR, int M, typename C>
-__device__ __forceinline__ void dft_twiddled(C (&x)[R], const C* __restrict__ tw, int i) {
-  if constexpr (R == 2) {
-    bfly<DIR>(x[0], x[1], ld_tw(&tw[i]));
-  } else if constexpr (R == 4) {
-    const C w1 = ld_tw(&tw[i]), w2 = ld_tw(&tw[2 * i]);
-    bfly<DIR>(x[0], x[2], w2);
-    bfly<DIR>(x[1], x[3], w2);
-    bfly<DIR>(x[0], x[1], w1);    // y0, y2
-    bfly_i<DIR>(x[2], x[3], w1);  // y1, y3
-    const C t = x[1];
-    x[1] = x[2];
-    x[2] = t;
-  } else {
-    static_assert(R == 8, "twiddled radix must be 2, 4 or 8");
-    const C w1 = ld_tw(&tw[i]), w2 = ld_tw(&tw[2 * i]), w4 = ld_tw(&tw[4 * i]), w1e = ld_tw(&tw[i + M / 8]);
+// tw: e^{-2 pi i m / M} table, i: index of w; NS: points transformed by the stages before, E: values per thread.
+template <int R, int DIR, int NS, int E>
+__device__ __forceinline__ void dft_twiddled(double2 (&x)[R], const double2* __restrict__ tw, int i) {
+  constexpr int H = R / 2;
+  constexpr bool SHORT = R == 8 || E == 4 || NS >= 64;
 #pragma unroll
-    for (int r = 0; r < 4; ++r) bfly<DIR>(x[r], x[r + 4], w4);
-    bfly<DIR>(x[0], x[2], w2);
-    bfly<DIR>(x[1], x[3], w2);
-    bfly_i<DIR>(x[4], x[6], w2);
-    bfly_i<DIR>(x[5], x[7], w2);
-    bfly<DIR>(x[0], x[1], w1);     // y0, y4
-    bfly_i<DIR>(x[2], x[3], w1);   // y2, y6
-    bfly<DIR>(x[4], x[5], w1e);    // y1, y5
-    bfly_i<DIR>(x[6], x[7], w1e);  // y3, y7
-    const C y4 = x[1], y1 = x[4], y6 = x[3], y3 = x[6];
-    x[1] = y1; x[3] = y3; x[4] = y4; x[6] = y6;
+  for (int r = 0; r < H; ++r) {
+    if (r > 0) x[r] = ctw<DIR>(x[r], ld_tw(&tw[r * i]));
+    bfly<DIR, SHORT>(x[r], x[r + H], ld_tw(&tw[(r + H) * i]));
+  }
+  if constexpr (R == 4) {
+    const double2 a = x[0], b = x[2], c = x[1], d = cmul_i<DIR>(x[3]);
+    x[0] = cadd(a, c); x[2] = csub(a, c); x[1] = cadd(b, d); x[3] = csub(b, d);
+  } else if constexpr (R == 8) {
+    dft8_rest<DIR>(x);
+  } else {
+    static_assert(R == 2, "twiddled radix must be 2, 4 or 8");
   }
 }
-// FP64 values take the fused form; the others multiply by the twiddles first.  A
-// forward and inverse pair of M = 128 then takes 37 FP64 instructions per point
-// instead of 43; with the multipliers as k (k/2M + c/M) and no moments where nobody
-// reads them, H phi on 128^3 complex128 went from 748 to 522 us (90% of its FP64
-// instructions' pipe time in both).
-template <typename C> struct FusedTwiddles { static constexpr bool value = false; };
-template <> struct FusedTwiddles<double2> { static constexpr bool value = true; };
 
 // Lanes of the calling warp that exist in this (1D) block.
 __device__ __forceinline__ unsigned block_warp_mask() {
@@ -269,8 +260,8 @@ __device__ __forceinline__ void fft_stages(C (&v)[E], C* sm, const SI& si, int t
     C x[R];
 #pragma unroll
     for (int r = 0; r < R; ++r) x[r] = v[b + r * NB];
-    if constexpr (NS > 1 && FusedTwiddles<C>::value && R <= 8) {
-      dft_twiddled<R, DIR, M>(x, tw, (j % NS) * (M / (NS * R)));
+    if constexpr (NS > 1 && std::is_same<C, double2>::value) {
+      dft_twiddled<R, DIR, NS, E>(x, tw, (j % NS) * (M / (NS * R)));
     } else {
       if constexpr (NS > 1) {
         const int k = j % NS;

@@ -692,6 +692,14 @@ template <typename T> struct MaxThreads { static constexpr int value = sizeof(T)
 // us instead of 522, energy and gradient on 512^2 469 instead of 452), so they stay out.
 template <int ROLE> constexpr bool kEarlyRole = ROLE == P_C1 || ROLE == P_C3 || ROLE == P_CFWD || ROLE == P_CCORE || ROLE == P_CINV;
 
+// Blocks per SM that the compiler must leave room for (0: as it likes; 1 would already
+// change what it takes): two in the FP64 H passes of 8 values per thread (256 threads).
+// Left alone it takes up to 158 registers, one block per SM, where two blocks with 64 to
+// 100 bytes of spills are faster: H phi on 256 x 256 x 32 complex128 570 -> 539 us, on
+// 64 x 256 x 128 567 -> 534, on 32 x 256 x 256 574 -> 539; on 128^3 531 both ways.
+template <typename TF, typename TS, int ROLE, int E> constexpr int kMinBlocks =
+    (std::is_same<TF, double>::value && std::is_same<TS, double>::value && (ROLE == P_HX || ROLE == P_HMID) && E == 8) ? 2 : 0;
+
 __device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
 
 template <typename To, typename From>
@@ -1167,7 +1175,8 @@ __device__ __forceinline__ void reduce_and_finish(const PassArgs& a, const Acc* 
 }
 
 template <typename TF, typename TS, typename TD, int M, int ROLE, int EV>
-__global__ void __launch_bounds__(MaxThreads<TF>::value < MaxThreads<TS>::value ? MaxThreads<TF>::value : MaxThreads<TS>::value) pass_x(PassArgs a) {
+__global__ void __launch_bounds__(MaxThreads<TF>::value < MaxThreads<TS>::value ? MaxThreads<TF>::value : MaxThreads<TS>::value,
+                                  kMinBlocks<TF, TS, ROLE, EV>) pass_x(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   if constexpr (kEarlyRole<ROLE>) pdl_wait();
   const Scal S = scal_of(a.ctl, a);
@@ -1181,7 +1190,7 @@ __global__ void __launch_bounds__(MaxThreads<TF>::value < MaxThreads<TS>::value 
 }
 
 template <typename T, int M, int ROLE, int EV>
-__global__ void __launch_bounds__(MaxThreads<T>::value) pass_s(PassArgs a) {
+__global__ void __launch_bounds__(MaxThreads<T>::value, kMinBlocks<T, T, ROLE, EV>) pass_s(PassArgs a) {
   extern __shared__ __align__(16) unsigned char smraw[];
   if constexpr (kEarlyRole<ROLE>) pdl_wait();
   const Scal S = scal_of(a.ctl, a);
