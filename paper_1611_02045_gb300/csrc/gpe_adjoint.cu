@@ -8,6 +8,10 @@
 // the pass kernels of the solver; this file adds the fused epilogues, the
 // inner products (FP64 sums, fixed order) and the scalar steps, which run on
 // the device so that the host reads scalars only at convergence checks.
+//
+// Every kernel here may be launched early (launch_early), so fields are read by coherent
+// loads (__ldcg): the kernel in front may still be writing r, y or q, and the caller's
+// phi and g_rho, when this one starts.
 #include "gpe_internal.h"
 
 namespace gpe {
@@ -165,9 +169,9 @@ __global__ void __launch_bounds__(kDotThreads) k_dots(const C* x0, const C* y0,
   y2 = after_wait(y2);
   double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    if (x0) { const C a = __ldg(x0 + i), b = __ldg(y0 + i); const double2 d = dconj_mul(a.x, a.y, b.x, b.y); v[0] += d.x; v[1] += d.y; }
-    if (x1) { const C a = __ldg(x1 + i), b = __ldg(y1 + i); v[2] += (double)a.x * b.x + (double)a.y * b.y; }  // real part
-    if (x2) { const C a = __ldg(x2 + i), b = __ldg(y2 + i); const double2 d = dconj_mul(a.x, a.y, b.x, b.y); v[4] += d.x; v[5] += d.y; }
+    if (x0) { const C a = __ldcg(x0 + i), b = __ldcg(y0 + i); const double2 d = dconj_mul(a.x, a.y, b.x, b.y); v[0] += d.x; v[1] += d.y; }
+    if (x1) { const C a = __ldcg(x1 + i), b = __ldcg(y1 + i); v[2] += (double)a.x * b.x + (double)a.y * b.y; }  // real part
+    if (x2) { const C a = __ldcg(x2 + i), b = __ldcg(y2 + i); const double2 d = dconj_mul(a.x, a.y, b.x, b.y); v[4] += d.x; v[5] += d.y; }
   }
   pdl_trigger();
   adj_reduce(v, red);
@@ -184,9 +188,10 @@ __global__ void __launch_bounds__(kDotThreads) k_hess_epi(const C* phi, const C*
   pdl_wait();
   phi = after_wait(phi);
   p = after_wait(p);
+  q = after_wait(q);
   double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const C f = __ldg(phi + i), d = __ldg(p + i);
+    const C f = __ldcg(phi + i), d = __ldcg(p + i);
     C h = q[i];
     const R u = f.x * f.x + f.y * f.y;
     const R s2x = f.x * f.x - f.y * f.y, s2y = R(2) * f.x * f.y;  // phi^2
@@ -214,11 +219,13 @@ __global__ void __launch_bounds__(kDotThreads) k_step(C* __restrict__ z, C* __re
   p = after_wait(p);
   q = after_wait(q);
   phi = after_wait(phi);
+  z = after_wait(z);
+  r = after_wait(r);
   if (S->stop) return;  // converged or broken down: leave z and r as they are
   const R a = R(S->a), cr = R(S->c_re), ci = R(S->c_im);
   double v[8] = {0, 0, 0, 0, 0, 0, 0, 0};
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const C d = __ldg(p + i), h = __ldg(q + i), f = __ldg(phi + i);
+    const C d = __ldcg(p + i), h = __ldcg(q + i), f = __ldcg(phi + i);
     C zz = z[i], rr = r[i];
     const R qx = h.x - (cr * f.x - ci * f.y), qy = h.y - (cr * f.y + ci * f.x);
     zz.x += a * d.x; zz.y += a * d.y;
@@ -239,7 +246,7 @@ __global__ void k_proj(const C* h_in, C* __restrict__ h_out, const C* phi, long 
   phi = after_wait(phi);
   const R cr = R(S->c_re), ci = R(S->c_im);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const C h = h_in[i], f = __ldg(phi + i);
+    const C h = h_in[i], f = __ldcg(phi + i);
     C o;
     o.x = h.x - (cr * f.x - ci * f.y);
     o.y = h.y - (cr * f.y + ci * f.x);
@@ -255,11 +262,12 @@ __global__ void k_dir(C* __restrict__ p, const C* y, const C* phi, long long n,
   pdl_wait();
   y = after_wait(y);
   phi = after_wait(phi);
+  p = after_wait(p);
   if (S->stop) return;
   const R cr = R(S->c_re), ci = R(S->c_im), b = R(S->beta);
   const bool keep = S->beta != 0.0;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const C h = __ldg(y + i), f = __ldg(phi + i);
+    const C h = __ldcg(y + i), f = __ldcg(phi + i);
     C o;
     o.x = h.x - (cr * f.x - ci * f.y);
     o.y = h.y - (cr * f.y + ci * f.x);
@@ -278,8 +286,8 @@ __global__ void k_density_rhs(const C* phi, const double* g_rho, C* __restrict__
   phi = after_wait(phi);
   g_rho = after_wait(g_rho);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const C f = __ldg(phi + i);
-    const R k = R(s * __ldg(g_rho + i));
+    const C f = __ldcg(phi + i);
+    const R k = R(s * __ldcg(g_rho + i));
     C o;
     o.x = k * f.x;
     o.y = k * f.y;
@@ -295,7 +303,7 @@ __global__ void k_dV_from_z(const C* phi, const C* z, double* __restrict__ gV, l
   phi = after_wait(phi);
   z = after_wait(z);
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-    const C f = __ldg(phi + i), q = __ldg(z + i);
+    const C f = __ldcg(phi + i), q = __ldcg(z + i);
     gV[i] = -weight * ((double)q.x * f.x + (double)q.y * f.y);
   }
 }

@@ -54,9 +54,15 @@ __host__ __device__ inline Num num(double d) {
 // keep plain launches.  Both calls do nothing in a kernel launched the plain way.
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;"); }
-// A field that the kernel before writes, where it is declared __restrict__: loads
-// through it may count as invariant to the compiler and move above pdl_wait, so they go
-// through the pointer that this returns after it.
+// What the kernel before writes is read by coherent loads: plain ones from a pointer
+// that is not both const and __restrict__, or __ldcg.  The non-coherent path (__ldg, and
+// what the compiler makes of const __restrict__) is for data that nobody writes while the
+// kernel runs, and an early kernel's run begins before its pdl_wait.  In P_C's passes
+// that covers s, which each pass stores as well; phi, r, V and the tables are older than
+// the kernel in front.
+// Where a pointer is const or __restrict__ its loads may also count as invariant to the
+// compiler and move above pdl_wait, so they go through the pointer that this returns
+// after it.
 template <typename T> __device__ __forceinline__ T* after_wait(T* p) {
   asm volatile("" : "+l"(p));
   return p;
