@@ -44,7 +44,7 @@ typedef enum {
   GPE_ERR_NOT_CONVERGED = 3, /* max_iter reached before the stopping rule held */
   GPE_ERR_NONFINITE = 4,     /* NaN/Inf met in a reduction */
   GPE_ERR_PRECOND = 5,       /* alpha + V + eta|phi|^2 <= 0 somewhere (P_V undefined) */
-  GPE_ERR_TIMEOUT = 6,       /* reserved: a bounded device wait gave up */
+  GPE_ERR_TIMEOUT = 6,       /* a bounded device wait gave up (never expected) */
   GPE_ERR_UNSUPPORTED = 7    /* configuration not supported by this build */
 } gpe_status;
 
@@ -174,7 +174,12 @@ gpe_status gpe_destroy(gpe_ctx* ctx);
 /* out = H_phi f = -1/2 Delta f + V f + eta |phi|^2 f - omega L_z f
  * (Section 2; discrete operators of eq. FFTdiscret).  phi_dev, f_dev,
  * out_dev: device fields in working precision; out may alias f but not phi.
- * Asynchronous.  Errors: GPE_ERR_ARG, GPE_ERR_CUDA. */
+ * Large complex64 3D fields take the dataflow of gpe_apply_H_batch for the x
+ * and y parts, so one such call runs at a time per context.
+ * Asynchronous.  Errors: GPE_ERR_ARG, GPE_ERR_CUDA; a bounded wait of a kernel
+ * that gives up is reported as GPE_ERR_TIMEOUT, once, by the next call on the
+ * context that returns host scalars (gpe_energy, gpe_energy_grad,
+ * gpe_tangent_solve, gpe_density_adjoint). */
 gpe_status gpe_apply_H(gpe_ctx* ctx, const void* phi_dev, const void* f_dev, void* out_dev);
 
 /* out_b = H_{phi_b} f_b for b = 0 .. nbatch-1 (the operator of gpe_apply_H,
@@ -198,10 +203,16 @@ gpe_status gpe_apply_H(gpe_ctx* ctx, const void* phi_dev, const void* f_dev, voi
  *    rows per CTA; E = 8 selects one field per cluster).
  * phi_dev, f_dev, out_dev: device arrays in working precision; f may equal
  * phi; out must not overlap phi or f.  Asynchronous.  A bounded wait of the
- * dataflow form that gives up (never expected) marks the context's API status
- * GPE_ERR_TIMEOUT.  Errors: GPE_ERR_ARG, GPE_ERR_UNSUPPORTED (other grids),
+ * dataflow form that gives up (never expected) is reported as for gpe_apply_H.
+ * Errors: GPE_ERR_ARG, GPE_ERR_UNSUPPORTED (other grids),
  * GPE_ERR_CUDA. */
 gpe_status gpe_apply_H_batch(gpe_ctx* ctx, int nbatch, const void* phi_dev, const void* f_dev, void* out_dev);
+
+/* Polls after which a wait of the dataflow form of gpe_apply_H and
+ * gpe_apply_H_batch (a column unit's for its plane's row units) gives up: 0 the
+ * default of 2^24 (seconds); < 0 at once, which shows how a program takes
+ * GPE_ERR_TIMEOUT.  Errors: GPE_ERR_ARG. */
+gpe_status gpe_set_wait_polls(gpe_ctx* ctx, int polls);
 
 /* out = P_C r = P_V^{1/2} P_Delta P_V^{1/2} r (eq. combinedP_12) with
  * P_Delta = (alpha - Delta/2)^{-1} (eq. PDelta) and
@@ -217,7 +228,7 @@ gpe_status gpe_precond(gpe_ctx* ctx, const void* phi_dev, const void* r_dev, dou
  * out[2] interaction eta/2 int |phi|^4, out[3] rotation -omega <phi, L_z phi>,
  * out[4] total E, out[5] lambda = <phi, H_phi phi>, out[6] lambda~ (eq. Opt_Alpha),
  * out[7] ||phi||^2.  phi is not normalised first.  Synchronises the stream.
- * Errors: GPE_ERR_ARG, GPE_ERR_CUDA. */
+ * Errors: GPE_ERR_ARG, GPE_ERR_CUDA, GPE_ERR_TIMEOUT (gpe_apply_H). */
 gpe_status gpe_energy(gpe_ctx* ctx, const void* phi_dev, double out[8]);
 
 /* Replace the context's potential and coupling constants without
@@ -245,7 +256,8 @@ gpe_status gpe_set_problem(gpe_ctx* ctx, const double* V, double eta, double ome
  * At a normalised critical point phi* (a ground state from gpe_pcg_solve) the
  * constraint terms vanish, so out[1], out[2] and grad_V are the derivatives
  * of the ground-state energy E*(V, eta, omega) itself (Hellmann-Feynman).
- * Synchronises the stream.  Errors: GPE_ERR_ARG, GPE_ERR_CUDA. */
+ * Synchronises the stream.  Errors: GPE_ERR_ARG, GPE_ERR_CUDA,
+ * GPE_ERR_TIMEOUT (gpe_apply_H). */
 gpe_status gpe_energy_grad(gpe_ctx* ctx, const void* phi_dev, void* grad_phi_dev, double* grad_V_dev, double out[5]);
 
 /* Tangent-space adjoint solve at a ground state: find z with <phi, z> = 0 and
@@ -269,7 +281,7 @@ gpe_status gpe_energy_grad(gpe_ctx* ctx, const void* phi_dev, void* grad_phi_dev
  * Synchronises the stream.  Errors: GPE_ERR_ARG, GPE_ERR_CUDA,
  * GPE_ERR_NOT_CONVERGED (max_iter reached; z holds the last iterate),
  * GPE_ERR_NONFINITE (K or P_C not positive -- phi is not a local minimum --
- * or a non-finite residual). */
+ * or a non-finite residual), GPE_ERR_TIMEOUT (gpe_apply_H; z is not valid). */
 gpe_status gpe_tangent_solve(gpe_ctx* ctx, const void* phi_dev, const void* rhs_dev, void* z_dev, double tol,
                              int max_iter, int* iters, double* rel_res);
 

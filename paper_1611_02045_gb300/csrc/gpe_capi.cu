@@ -52,6 +52,7 @@ struct PrecBufs {
 struct Pinned {
   Ctl ctl;
   AdjScalars adj;
+  int wait_status;  // ctl_api->status
   TfState tf;
   VCheck v;
 };
@@ -83,6 +84,7 @@ struct gpe_ctx {
   int hflow_cap = 0;
   int* hflow_old[24] = {};  // outgrown counters (sizes at least double): a graph captured with them may still run
   int hflow_nold = 0;
+  int wait_polls = 0;    // polls of its waits (gpe_set_wait_polls)
   int hbatch_E = 8;      // values per thread of gpe_apply_H_batch's cluster kernel (plan mode 3):
                          // 16 (streaming form) by default in single precision for n >= 64
   Pinned* pinned = nullptr;
@@ -494,6 +496,7 @@ static gpe_status try_flow(gpe_ctx* c, int nplanes, long long vstride, const voi
   a.ctr = c->hflow_ctr;
   a.ctr_cap = c->hflow_cap;
   a.status = &c->ctl_api->status;
+  a.polls = c->wait_polls;
   GPE_CU(c, launch_h_batch_flow(a, c->st, used));
   return GPE_OK;
 }
@@ -573,6 +576,23 @@ extern "C" gpe_status gpe_apply_H_batch(gpe_ctx* c, int nbatch, const void* phi,
   return GPE_OK;
 }
 
+// The kernels of the API calls leave GPE_ERR_TIMEOUT in the API control block when a
+// bounded wait gives up, which asynchronous calls cannot return: every call that copies
+// the block, or its status, to the host passes the status here.  It is reported once.
+static gpe_status check_waits(gpe_ctx* c, int status) {
+  if (status == GPE_OK) return GPE_OK;
+  GPE_CU(c, cudaMemsetAsync(&c->ctl_api->status, 0, sizeof(int), c->st));
+  GPE_CU(c, cudaMemsetAsync(&c->ctl_api->done, 0, sizeof(int), c->st));
+  c->err = "a bounded device wait gave up: results since the last call that synchronised are not valid";
+  return GPE_ERR_TIMEOUT;
+}
+
+extern "C" gpe_status gpe_set_wait_polls(gpe_ctx* c, int polls) {
+  if (!c) return GPE_ERR_ARG;
+  c->wait_polls = polls;
+  return GPE_OK;
+}
+
 extern "C" gpe_status gpe_energy(gpe_ctx* c, const void* phi, double out[8]) {
   if (!c) return GPE_ERR_ARG;
   if (!phi || !out) { c->err = "null pointer"; return GPE_ERR_ARG; }
@@ -582,6 +602,7 @@ extern "C" gpe_status gpe_energy(gpe_ctx* c, const void* phi, double out[8]) {
   GPE_CU(c, cudaMemcpyAsync(&c->pinned->ctl, c->ctl_api, sizeof(Ctl), cudaMemcpyDeviceToHost, c->st));
   GPE_CU(c, cudaStreamSynchronize(c->st));
   const Ctl& h = c->pinned->ctl;
+  if ((s = check_waits(c, h.status)) != GPE_OK) return s;
   out[0] = h.kin; out[1] = h.pot; out[2] = 0.5 * c->prob.eta * h.U0; out[3] = h.rot;
   out[4] = h.E; out[5] = h.lam; out[6] = h.alpha; out[7] = h.norm2;
   return GPE_OK;
@@ -616,6 +637,7 @@ extern "C" gpe_status gpe_energy_grad(gpe_ctx* c, const void* phi, void* grad_ph
   GPE_CU(c, cudaMemcpyAsync(&c->pinned->ctl, c->ctl_api, sizeof(Ctl), cudaMemcpyDeviceToHost, c->st));
   GPE_CU(c, cudaStreamSynchronize(c->st));
   const Ctl& h = c->pinned->ctl;
+  if ((s = check_waits(c, h.status)) != GPE_OK) return s;
   out[0] = h.E;
   out[1] = 0.5 * h.U0;  // d/d eta of eta/2 int |phi|^4
   out[2] = -h.Lz;       // d/d omega of -omega <phi, L_z phi>
@@ -788,6 +810,7 @@ static gpe_status tangent_solve(gpe_ctx* c, const void* phi, const void* rhs, vo
   if (s != GPE_OK) return s;
   GPE_CU(c, cudaMemcpyAsync(&c->pinned->ctl, c->ctl_api, sizeof(Ctl), cudaMemcpyDeviceToHost, st));
   GPE_CU(c, cudaStreamSynchronize(st));
+  if ((s = check_waits(c, c->pinned->ctl.status)) != GPE_OK) return s;
   const double lam = c->pinned->ctl.lam, alpha = c->pinned->ctl.alpha;
   if (!std::isfinite(lam) || !(alpha > 0.0)) { c->err = "phi gives a non-finite lambda or a shift <= 0"; return GPE_ERR_NONFINITE; }
   AdjScalars s0;
@@ -811,8 +834,11 @@ static gpe_status tangent_solve(gpe_ctx* c, const void* phi, const void* rhs, vo
   for (;;) {
     if (it % kAdjCheckEvery == 0 || it >= max_iter) {
       GPE_CU(c, cudaMemcpyAsync(&c->pinned->adj, S, sizeof(hs), cudaMemcpyDeviceToHost, st));
+      if (prec == 0)  // complex128 passes wait for nothing
+        GPE_CU(c, cudaMemcpyAsync(&c->pinned->wait_status, &c->ctl_api->status, sizeof(int), cudaMemcpyDeviceToHost, st));
       GPE_CU(c, cudaStreamSynchronize(st));
       hs = c->pinned->adj;
+      if (prec == 0 && (s = check_waits(c, c->pinned->wait_status)) != GPE_OK) return s;
       if (hs.stop || it >= max_iter) break;
     }
     // q = P K p;  a = Re<r, y> / Re<p, q>;  z += a p;  r -= a q

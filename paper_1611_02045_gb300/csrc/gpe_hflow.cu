@@ -42,6 +42,10 @@
 // Counters (ctr, owned by the context, zero between launches): ctr[0] ticket,
 // ctr[1] blocks finished, ctr[2 + b] x units of plane b done.  The last block to
 // finish zeroes them, so no separate reset runs before the next launch.
+//
+// A wait that gives up marks *status, leaves its unit's sum out and its block takes no
+// further unit: the launch ends (later waits on what the block dropped give up as well),
+// out is not valid and the next launch starts from zero counters again.
 #include <cuda_runtime.h>
 
 #include <atomic>
@@ -82,6 +86,7 @@ struct FlowArgs {
   float2* out;
   int* ctr;     // [0] ticket, [1] blocks finished, [2 + b] x units done of plane b
   int* status;  // set to GPE_ERR_TIMEOUT (6) when a bounded wait gives up (may be null)
+  long long polls;  // of a y unit's wait for its plane's x units before it gives up
 };
 
 // Ticket u -> (type 0 = x unit / 1 = y unit, plane, unit of the plane), NU units of
@@ -193,7 +198,7 @@ __device__ __forceinline__ void dft_col(float2 (&v)[16], float2* tile, int t, in
 
 template <int MX, int MY, bool SAME>
 __global__ void __launch_bounds__(256, 2)
-    h_batch_flow(FlowArgs a, const __grid_constant__ CUtensorMap tmF, const __grid_constant__ CUtensorMap tmO) {
+    h_batch_flow(const __grid_constant__ FlowArgs a, const __grid_constant__ CUtensorMap tmF, const __grid_constant__ CUtensorMap tmO) {
   using C = float2;
   using LX = FlowLine<MX>;
   using LY = FlowLine<MY>;
@@ -344,12 +349,14 @@ __global__ void __launch_bounds__(256, 2)
         // the plane's x units must have stored t before the TMA adds A_y f to it
         long long n = 0;
         if (early < NU)
-          while (ld_acquire_gpu(a.ctr + 2 + fld) < NU && n < kTmaWaitLimit) ++n;
-        if (n >= kTmaWaitLimit) ok = false;
+          while (ld_acquire_gpu(a.ctr + 2 + fld) < NU && n < a.polls) ++n;
+        if (n >= a.polls) ok = false;
         asm volatile("fence.proxy.async;" ::: "memory");  // generic stores of out -> the TMA's adds
+        if (ok) {
 #pragma unroll
-        for (int b = 0; b < LY::NBOX; ++b)
-          tma_reduce_add_3d(&tmO, st + b * 16 * MY, 32 * (blk * LY::NBOX + b), 0, fld);
+          for (int b = 0; b < LY::NBOX; ++b)
+            tma_reduce_add_3d(&tmO, st + b * 16 * MY, 32 * (blk * LY::NBOX + b), 0, fld);
+        }
         asm volatile("cp.async.bulk.commit_group;" ::: "memory");
         asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");  // tiles read before the refill
       }
@@ -477,6 +484,7 @@ cudaError_t launch_h_batch_flow(const FlowHArgs& a, cudaStream_t st, bool* used)
   fa.out = static_cast<float2*>(a.out);
   fa.ctr = a.ctr;
   fa.status = a.status;
+  fa.polls = a.polls == 0 ? kTmaWaitLimit : (a.polls < 0 ? 0 : a.polls);
   switch (a.mx) {
     case 64: return launch_flow_y<64>(a.my, fa, tmF, tmO, st, used);
     case 128: return launch_flow_y<128>(a.my, fa, tmF, tmO, st, used);

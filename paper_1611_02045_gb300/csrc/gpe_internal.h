@@ -255,6 +255,7 @@ struct FlowHArgs {
   int* ctr;     // zeroed counters, at least h_batch_flow_counters(nbatch) ints
   int ctr_cap;
   int* status;  // device int set to GPE_ERR_TIMEOUT when a bounded wait gives up (or null)
+  int polls;    // of a y unit's wait before it gives up: 0 the default, < 0 none
 };
 cudaError_t launch_h_batch_flow(const FlowHArgs& a, cudaStream_t st, bool* used);
 size_t h_batch_flow_counters(int nbatch);

@@ -65,7 +65,7 @@ EXPORTED = ("gpe_solve_opts_default", "gpe_create", "gpe_destroy", "gpe_apply_H"
             "gpe_energy", "gpe_set_problem", "gpe_energy_grad", "gpe_tangent_solve", "gpe_density_adjoint",
             "gpe_pcg_solve", "gpe_last_error", "gpe_batch_create", "gpe_batch_solve", "gpe_batch_destroy",
             "gpe_batch_last_error", "gpe_autotune", "gpe_set_plan", "gpe_get_plan", "gpe_batch_autotune",
-            "gpe_thomas_fermi", "gpe_interpolate", "gpe_alu_peak")
+            "gpe_thomas_fermi", "gpe_interpolate", "gpe_alu_peak", "gpe_set_wait_polls")
 MODE_NAMES = ("complex64", "fp64", "refinement")
 _STRING_RETURNING = ("gpe_last_error", "gpe_batch_last_error")
 
@@ -105,6 +105,7 @@ def lib():
         L.gpe_batch_autotune.argtypes = [vp, C.c_int]
         L.gpe_thomas_fermi.argtypes = [vp, vp, C.POINTER(C.c_double)]
         L.gpe_interpolate.argtypes = [vp, vp, vp, vp]
+        L.gpe_set_wait_polls.argtypes = [vp, C.c_int]
         L.gpe_alu_peak.argtypes = [C.c_int, vp, C.POINTER(C.c_double)]
         for name in EXPORTED:
             if name not in _STRING_RETURNING:
@@ -182,6 +183,10 @@ class Context:
 
     def apply_H_batch(self, nbatch, phi, f, out):
         return self._check(lib().gpe_apply_H_batch(self._ctx, int(nbatch), _addr(phi), _addr(f), _addr(out)))
+
+    def set_wait_polls(self, polls):
+        """gpe_set_wait_polls: polls of the dataflow's waits (0 the default, < 0 give up at once)."""
+        return self._check(lib().gpe_set_wait_polls(self._ctx, int(polls)))
 
     def precond(self, phi, r, alpha, out):
         return self._check(lib().gpe_precond(self._ctx, _addr(phi), _addr(r), float(alpha), _addr(out)))
