@@ -414,7 +414,12 @@ gpe_status gpe_autotune(gpe_ctx* ctx, int iters, int use_cache, gpe_tune_report*
 /* Set / read the plan of (mode, axis).  gpe_set_plan rejects plans the kernels
  * cannot run (E not 4 or 8, E = 4 below M = 32, width not a power of two, more
  * threads than the mode's kernels allow, too much shared memory, more blocks
- * than the context's reduction buffers) with GPE_ERR_ARG.  Mode 3, axis 0 is
+ * than the context's reduction buffers) with GPE_ERR_ARG.  gpe_apply_H on
+ * complex64 fields runs the passes of mode 0 as they are set here; where no
+ * plan has been set (or gpe_autotune has chosen the plans since), it takes one
+ * cluster for square 2D fields of 32 to 128 points per side, and the dataflow
+ * of gpe_apply_H_batch in place of the x and y passes for 3D fields of at least
+ * 2^22 points with sides of 64, 128 or 256.  Mode 3, axis 0 is
  * the kernel of gpe_apply_H_batch: E = 8 (one field per cluster, 16 rows per
  * CTA) or E = 16 (single precision, n >= 64) with width 16 (the dataflow form
  * where it applies, else the streaming form with a cluster of n/16 CTAs) or

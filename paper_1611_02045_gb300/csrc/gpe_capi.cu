@@ -78,6 +78,7 @@ struct gpe_ctx {
   double* log_dev = nullptr;
   int log_dev_cap = 0;
   PassPlan mplan[3][3];  // plan used per launch mode [mode][axis] (plan_axis, or the tuner's choice)
+  bool plan_set[3] = {false, false, false};  // complex64 plans of the caller's own (gpe_set_plan), per axis
   int partials_cap = 0;  // blocks the reduction partials buffer holds
   int hbatch_rows = 16;  // rows per CTA of its streaming form (plan mode 3 width: 16 or 32)
   int* hflow_ctr = nullptr;  // counters of gpe_apply_H_batch's dataflow form (zero between launches)
@@ -504,7 +505,8 @@ static gpe_status try_flow(gpe_ctx* c, int nplanes, long long vstride, const voi
 static gpe_status run_H(gpe_ctx* c, int prec, const void* phi, const void* f, void* out, Ctl* ctl,
                         HWant want = H_AND_MOMENTS) {
   bool flowed = false;
-  if (prec == 0 && want == H_ONLY && c->dim == 3 && flow_pays(c, c->N)) {
+  // (in place of the x and y passes, unless the caller planned one of them)
+  if (prec == 0 && want == H_ONLY && c->dim == 3 && flow_pays(c, c->N) && !c->plan_set[0] && !c->plan_set[1]) {
     const gpe_status s = try_flow(c, c->n[2], (long long)c->n[0] * c->n[1], phi, f, c->pb[0].t, &flowed);
     if (s != GPE_OK) return s;
   }
@@ -544,8 +546,9 @@ static ClusterHArgs cluster_args(const gpe_ctx* c, int prec, int nbatch, const v
 extern "C" gpe_status gpe_apply_H(gpe_ctx* c, const void* phi, const void* f, void* out) {
   if (!c) return GPE_ERR_ARG;
   if (!phi || !f || !out) { c->err = "null field pointer"; return GPE_ERR_ARG; }
-  if (c->work == 0 && c->dim == 2 && c->n[0] == c->n[1] && c->n[0] >= 32 && c->n[0] <= 128) {
-    // one launch for a small square field, in one cluster (which reads all of f before it
+  if (c->work == 0 && c->dim == 2 && c->n[0] == c->n[1] && c->n[0] >= 32 && c->n[0] <= 128 && !c->plan_set[0] &&
+      !c->plan_set[1]) {
+    // one launch for a small square field whose passes the caller has not planned, in one cluster (which reads all of f before it
     // writes: out may be f).  Device time against the two passes: 32^2 4.7 / 6.7 us, 64^2
     // 6.1 / 8.4, 128^2 8.5 / 9.4, 256^2 15.1 / 9.5; in complex128 the FP64 pipes of the
     // cluster's few SMs are the limit (32^2 27 / 17 us)
@@ -1246,6 +1249,7 @@ extern "C" gpe_status gpe_set_plan(gpe_ctx* c, int mode, int axis, int E, int wi
   if (!make_plan(c, mode, axis, E, width, pl)) { c->err = "plan not supported for this grid and mode"; return GPE_ERR_ARG; }
   GPE_CU(c, cudaStreamSynchronize(c->st));
   c->mplan[mode][axis] = pl;
+  if (mode == 0) c->plan_set[axis] = true;
   plans_changed(c, mode);
   return GPE_OK;
 }
@@ -1386,6 +1390,8 @@ extern "C" gpe_status gpe_autotune(gpe_ctx* c, int iters, int use_cache, gpe_tun
       r.E[mode][ax] = c->mplan[mode][ax].E;
       r.width[mode][ax] = ax == 0 ? c->mplan[mode][ax].lpb : c->mplan[mode][ax].tx;
     }
+    if (mode == 0)
+      for (auto& own : c->plan_set) own = false;  // the plans are the tuner's now
     plans_changed(c, mode);
   }
   if (rep) *rep = r;
