@@ -361,7 +361,6 @@ __global__ void __launch_bounds__(512) pass_xc_bulk(PassArgs a) {
   extern __shared__ __align__(128) unsigned char smraw[];
   __shared__ __align__(8) unsigned long long bar[2];
   __shared__ PassArgs sa[2];  // the unit body's arguments, pointed at stage s
-  if constexpr (kEarlyRole<ROLE>) pdl_wait();
   if (a.solver && a.ctl->done) return;
   const Scal S = scal_of(a.ctl, a);
   const int lpb = a.lpb;
@@ -443,7 +442,6 @@ __global__ void __launch_bounds__(512) pass_xc_bulk(PassArgs a) {
     if (threadIdx.x == 0) store(u, s);
   }
   if (threadIdx.x == 0) asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
-  if constexpr (kEarlyRole<ROLE>) pdl_trigger();
   reduce_and_finish<ROLE>(a, acc);
 }
 // Tensor map over a complex64 field [nz][ny][nx] (8-byte elements), boxes of
@@ -614,7 +612,8 @@ cudaError_t launch_xc_one(const PassArgs& a0, cudaStream_t st, bool* used) {
   // at least two units per block, and no more blocks than the plan's (the reduction partials hold those)
   if (a.nblocks < 2 * grid || grid > a0.nblocks) return cudaSuccess;
   *used = true;
-  return launch_early(kEarlyRole<ROLE> && a.early && !a.solver, kern, grid, threads, smem, st, a);
+  kern<<<(unsigned)grid, threads, smem, st>>>(a);  // inside a solve: launched plainly
+  return cudaGetLastError();
 }
 
 template <int ROLE>
