@@ -353,10 +353,10 @@ gpe_status gpe_pcg_solve(gpe_ctx* ctx, void* phi_inout, const gpe_solve_opts* op
  * memory already exhausted -- and so cannot create a context.
  *
  * Computes the same out = H_phi f as gpe_apply_H with the same pass kernels,
- * under default plans (a context's tuned plans may sum in another order, so
- * results agree to rounding), but takes the problem directly and keeps its
- * intermediate field, grid tables, reduction partials and control block in
- * one fixed static device array of libgpe (about 17 MiB, held by every GPU
+ * under plans of its own (a context's plans, its cluster and its dataflow
+ * forms sum in another order, so results agree to rounding), but takes the
+ * problem directly and keeps its intermediate field, grid tables and control
+ * block in one fixed static device array of libgpe (16 MiB, held by every GPU
  * that loads the library until the process exits).  It calls no
  * cudaMalloc/cudaFree and no allocating library.
  *  prob    : as for gpe_create; prob->prec selects the element types.
@@ -367,9 +367,8 @@ gpe_status gpe_pcg_solve(gpe_ctx* ctx, void* phi_inout, const gpe_solve_opts* op
  *  stream  : cudaStream_t ordering the work (NULL = legacy default stream).
  *  err, err_len : optional buffer for a message (NUL-terminated), may be NULL.
  * Limits: N * sizeof(element) <= 16 MiB, i.e. at most 2^20 complex128 or 2^21
- * complex64 points; and at most 8192 thread blocks in any axis's pass (the
- * partials the array holds), which excludes some flat 3D grids such as
- * 512 x 8 x 512.  Both are checked before any work is queued: such calls
+ * complex64 points; and at most 8192 thread blocks in any axis's pass, which
+ * excludes some flat 3D grids such as 512 x 8 x 512.  Both are checked before any work is queued: such calls
  * return GPE_ERR_UNSUPPORTED with the sizes in err and leave out untouched.
  * Each call outside a stream capture looks up the array's device address on
  * the current device (cudaGetSymbolAddress); a call inside a capture uses the

@@ -272,11 +272,12 @@ static cudaError_t upload_tables(gpe_ctx* c, PrecBufs& b) {
 
 // Take the potential V (float64, host or device): check that it is finite, record
 // its extremes and write it in every precision in use (float32, float64,
-// double-single).  A potential that is not finite changes nothing.  Two kernels on
-// the legacy default stream, which orders them after the caller's work on blocking
-// streams as a plain copy would be, and one host synchronisation: V may be changed
-// or freed when this returns.  The check reads V once and the conversion once more
-// (from L2), where a copy to the host, a loop over it and an allocation took most
+// double-single).  A potential that is not finite changes nothing.  Three kernels
+// (reset, check, conversion) on the legacy default stream, which orders them after the
+// caller's work on blocking streams as a plain copy would be, and one host
+// synchronisation: V may be changed or freed when this returns.  The check reads V once
+// and the conversion once more (from L2 where V fits), where a copy to the host, a loop
+// over it and an allocation took most
 // of a set_problem call (complex128 contexts: 256^2 104 -> 30 us, 128^3 2529 -> 37 us).
 static bool readable_here(const double* p) {  // by a kernel: this device's own memory, aligned
   cudaPointerAttributes at{};

@@ -29,23 +29,21 @@ namespace {
 // Capacity of the intermediate field: 16 MiB = 2^20 complex128 or 2^21
 // complex64 points (512^2, 1024^2 in complex64, 128 x 128 x 64, ...).
 constexpr size_t kFieldBytes = size_t(16) << 20;
-// Control block, ticket, reduction partials (up to kMaxBlocks blocks) and
-// tables (three axes of at most 512 points).
-constexpr int kMaxBlocks = 8192;
+// In front of it the control block and the tables (three axes of at most 512 points).
+// The passes run without reductions (H phi as a plain operator), so no ticket and no
+// partials are kept.
+constexpr int kMaxBlocks = 8192;  // per pass: the documented limit of the interface
 constexpr size_t kCtlOff = 0;
-constexpr size_t kTicketOff = 4096;
-constexpr size_t kPartialsOff = 8192;
-constexpr size_t kPartialsBytes = size_t(kMaxBlocks) * kMaxMoments * sizeof(double);
-constexpr size_t kTablesOff = kPartialsOff + kPartialsBytes;
+constexpr size_t kTablesOff = 4096;
 constexpr size_t kTablesBytes = size_t(3) * 4 * 512 * sizeof(double);  // xi, xc, tw(re, im) per axis
 constexpr size_t kFieldOff = (kTablesOff + kTablesBytes + 255) & ~size_t(255);
 constexpr size_t kScratchBytes = kFieldOff + kFieldBytes;
-static_assert(sizeof(Ctl) <= kTicketOff, "control block must fit before the ticket");
+static_assert(sizeof(Ctl) <= kTablesOff, "control block must fit before the tables");
 
 constexpr int kMaxDevices = 64;
 void* g_scratch_addr[kMaxDevices] = {nullptr};  // device address of g_scratch, per device
 
-constexpr int kTargetBlocks = 2 * 152;
+constexpr int kTargetBlocks = 2 * 152;  // blocks wanted per pass
 
 void set_err(char* err, size_t len, const char* msg) {
   if (err && len > 0) std::snprintf(err, len, "%s", msg);
@@ -112,8 +110,8 @@ extern "C" gpe_status gpe_apply_H_noalloc(const gpe_problem* prob, const void* V
     return GPE_ERR_UNSUPPORTED;
   }
 
-  // Pass plans for every axis, checked before anything is queued: the same
-  // rules as a context's default plans, with the FP64 thread cap.
+  // Pass plans for every axis, checked before anything is queued: E = 8, the widest
+  // blocks up to the FP64 thread cap, halved while an axis has fewer than 304 of them.
   const int maxT = 256;
   int lpb = maxT / (n[0] / 8);
   if (lpb < 1) lpb = 1;
@@ -133,8 +131,8 @@ extern "C" gpe_status gpe_apply_H_noalloc(const gpe_problem* prob, const void* V
   for (int ax = 0; ax < prob->dim; ++ax) {
     if (blocks_ax[ax] > kMaxBlocks) {
       char msg[160];
-      std::snprintf(msg, sizeof(msg), "axis %d needs %lld thread blocks; the scratch holds reduction partials for "
-                    "at most %d", ax, blocks_ax[ax], kMaxBlocks);
+      std::snprintf(msg, sizeof(msg), "axis %d needs %lld thread blocks; the limit is %d", ax, blocks_ax[ax],
+                    kMaxBlocks);
       set_err(err, err_len, msg);
       return GPE_ERR_UNSUPPORTED;
     }
