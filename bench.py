@@ -452,11 +452,12 @@ def main():
                      "flop_model": "5 M log2 M per line transform x 6 transforms + 20 per point",
                      "peak_source": "gpe_alu_peak(fp64 fma), measured in this run"}
 
-    # ---------------- H phi on one 256x256x512 complex64 field (beyond L2): the pass kernels ----------------
-    # gpe_apply_H = x pass (phi, V in; t out), y and z passes (f, t in; t / H phi out), each a
-    # TMA-fed persistent kernel; algorithmic bytes 20 per point for the operator (read phi and V,
-    # write H phi) and 68 per point summed over the three passes (20 + 24 + 24).  Per-pass DRAM figures: the ncu
-    # summary profiles/fft_passes_256x256x512_c64.md.
+    # ---------------- H phi on one 256x256x512 complex64 field (beyond L2) ----------------
+    # By default the x and y parts run as one dataflow launch over the z planes (phi and V in, t
+    # out: 20 bytes per point, the planes' y parts staying in L2), then the z pass (f and t in, H phi
+    # out: 24).  With a plan set for an axis the three passes run: x (20), y and z (24 each), TMA-fed
+    # persistent kernels whose DRAM figures are in profiles/fft_passes_256x256x512_c64.md.  The
+    # operator itself needs 20 bytes per point (read phi and V, write H phi).
     fftpass = None
     if rank == 0 and not args.no_fftpass:
         nf3, Lf3 = (256, 256, 512), (8.0, 8.0, 8.0)
@@ -465,24 +466,31 @@ def main():
             gf = torch.Generator(device=dev).manual_seed(5)
             xf = torch.randn(Nf3, dtype=torch.complex64, device=dev, generator=gf)
             yf = torch.empty_like(xf)
-            for _ in range(3):
-                cf3.apply_H(xf, xf, yf)
-            tf = []
-            for _ in range(10):
-                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-                a.record(stream)
-                cf3.apply_H(xf, xf, yf)
-                b.record(stream)
-                b.synchronize()
-                tf.append(a.elapsed_time(b))
+
+            def time_f3(bytes_per_point, kernels):
+                for _ in range(3):
+                    cf3.apply_H(xf, xf, yf)
+                tf = []
+                for _ in range(10):
+                    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                    a.record(stream)
+                    cf3.apply_H(xf, xf, yf)
+                    b.record(stream)
+                    b.synchronize()
+                    tf.append(a.elapsed_time(b))
+                msf = statistics.median(tf)
+                gbs = bytes_per_point * Nf3 / (msf * 1e-3) / 1e9
+                return {"ms_per_call": msf, "operator_gbs": 20.0 * Nf3 / (msf * 1e-3) / 1e9,
+                        "bytes_per_point": bytes_per_point, "passes_gbs": gbs, "passes_frac": gbs / peak,
+                        "kernels": kernels}
+
+            fftpass = {"field": "256x256x512 complex64 (268 MB)",
+                       **time_f3(20 + 24, "h_batch_flow<256,256> on 512 planes, pass_s_tma<512,8,HMID>")}
+            cf3.set_plan(0, 0, *cf3.get_plan(0, 0))  # the caller's own plan, though the same: the passes run
+            fftpass["three_passes"] = time_f3(20 + 24 + 24, "pass_hx_bulk<256,8>, pass_s_tma<256,8,HMID>, "
+                                                            "pass_s_tma<512,8,HMID>")
+            fftpass["per_pass"] = "profiles/fft_passes_256x256x512_c64.md"
             del xf, yf
-        msf = statistics.median(tf)
-        fftpass = {"field": "256x256x512 complex64 (268 MB)", "ms_per_call": msf,
-                   "operator_gbs": 20.0 * Nf3 / (msf * 1e-3) / 1e9,
-                   "passes_gbs": 68.0 * Nf3 / (msf * 1e-3) / 1e9,
-                   "passes_frac": 68.0 * Nf3 / (msf * 1e-3) / 1e9 / peak,
-                   "kernels": "pass_hx_bulk<256,8>, pass_s_tma<256,8,HMID>, pass_s_tma<512,8,HMID>",
-                   "per_pass": "profiles/fft_passes_256x256x512_c64.md"}
 
     # ---------------- secondary: the 128^3 workload ----------------
     secondary = None
