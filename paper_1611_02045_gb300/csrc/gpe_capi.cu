@@ -139,7 +139,10 @@ static bool is_device_ptr(const void* p) {
 //  * width: the widest block up to the thread cap, halved while the axis has fewer
 //    than 128 blocks and the block more than one warp: blocks below a warp waste
 //    lanes, and every block costs a ticket and a partial (32^3 with blocks of 8
-//    threads: 158 us per complex64 iteration against 79 with these widths).
+//    threads: 158 us per complex64 iteration against 79 with these widths).  Strided
+//    tiles have up to 16 columns, those of lines below 64 points up to 128 threads: with
+//    16 columns the z pass of 256 x 128 x 16 has 2048 blocks of a warp, whose partials
+//    the last one sums alone (gpe_energy, complex64: 93 us against 57 with 64 columns).
 static void plan_axis(const gpe_ctx* c, int mode, int axis, PassPlan& pl) {
   const int M = c->n[axis];
   const bool few = c->N <= (1ll << 17);
@@ -152,7 +155,8 @@ static void plan_axis(const gpe_ctx* c, int mode, int axis, PassPlan& pl) {
                                     : (axis == 1 ? (c->dim == 3 ? c->n[2] : 1) : c->n[1]);
   int w = maxT / Tl;
   if (w < 1) w = 1;
-  if (axis > 0 && w > 16) w = 16;
+  const int wide = Tl < 8 ? 128 / Tl : 16;
+  if (axis > 0 && w > wide) w = wide;
   while (w > 1 && w > (axis == 0 ? outer : per)) w >>= 1;
   auto blocks = [&](int v) { return axis == 0 ? outer / v : per / v * outer; };
   const int least = axis == 0 ? 1 : (mode == 0 ? 4 : 2);  // strided tiles: 32-byte sectors

@@ -247,15 +247,36 @@ __device__ __forceinline__ double total(Acc x, double weight, int k) {
 template <int K, unsigned MAXMASK, typename Src, typename Nb, typename Sink>
 __device__ __forceinline__ void sum_partials(Src src, Nb nb, Acc* red_sm, Sink sink) {
   constexpr int lg = Slots<K>::lg, P = Slots<K>::P, U = 16;
+  static_assert(16 * K <= kRedSlots, "one row of slots per thread of a block below a warp");
   if (blockDim.x < 32) {
+    // a thread takes every blockDim-th block, all slots' loads in flight at once: one
+    // slot per thread, one load at a time, took 360 us over the 1024 blocks of 16 threads
+    // of a z pass of 128 x 128 x 8
+    Acc t[K];
+    int n[K], most = 0;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+      t[k] = Acc{0.0f, 0.0f};
+      n[k] = nb(k);
+      most = n[k] > most ? n[k] : most;
+    }
+#pragma unroll 2
+    for (int b = threadIdx.x; b < most; b += blockDim.x) {
+      float2 x[K];
+#pragma unroll
+      for (int k = 0; k < K; ++k)
+        x[k] = b < n[k] ? __ldcg(reinterpret_cast<const float2*>(src(k)) + (size_t)b * kMaxMoments) : make_float2(0.0f, 0.0f);
+#pragma unroll
+      for (int k = 0; k < K; ++k) t[k] = red_op<MAXMASK>(t[k], Acc{x[k].x, x[k].y}, k);
+    }
+    __syncthreads();  // earlier readers of red_sm
+#pragma unroll
+    for (int k = 0; k < K; ++k) red_sm[threadIdx.x * K + k] = t[k];
+    __syncthreads();
     for (int k = threadIdx.x; k < K; k += blockDim.x) {
-      const float2* p = reinterpret_cast<const float2*>(src(k));
-      Acc t{0.0f, 0.0f};
-      for (int b = 0; b < nb(k); ++b) {
-        const float2 x = __ldcg(p + (size_t)b * kMaxMoments);
-        t = red_op<MAXMASK>(t, Acc{x.x, x.y}, k);
-      }
-      sink(k, t);
+      Acc r = red_sm[k];
+      for (int j = 1; j < (int)blockDim.x; ++j) r = red_op<MAXMASK>(r, red_sm[j * K + k], k);
+      sink(k, r);
     }
     return;
   }
