@@ -778,7 +778,14 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
     const bool retract = S.retract;
     const CD* __restrict__ p = static_cast<const CD*>(a.p);
     CS* __restrict__ phi_out = static_cast<CS*>(a.phi_out);
-    CD pq[E];
+    // ONE: the second field -- p in a solve, the operand f of an API call -- has the state's
+    // type and comes through one pointer into v, all loads of the block in flight together.
+    // A choice per element put f behind phi: 0.5 to 1 us of L2 latency in H phi with f != phi
+    // (device time on 512^2 complex64 10.4 -> 8.9 us, 64 x 128 6.8 -> 4.8).  Complex64 passes
+    // keep the operand over the transforms (512^2: 9.3 with f read again behind them); FP64
+    // passes, short of registers, read it again.
+    constexpr bool ONE = std::is_same<TS, TD>::value && !RES, KEEP = ONE && std::is_same<TS, float>::value;
+    CD pq[ONE && !KEEP ? 1 : E];  // p of a refinement; the operand kept
     if constexpr (RES) {
       const TS cc = num_as<TS>(S.cc), ss = num_as<TS>(S.ss);
 #pragma unroll
@@ -794,14 +801,23 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
         vv[q] = V[g];
         v[q] = cconv<TF>(x);
       }
-    } else {
+    } else if constexpr (ONE) {
+      const CS* __restrict__ second = a.solver ? p : f;
+#pragma unroll
+      for (int q = 0; q < E; ++q) {
+        const long long g = base + t + q * Tl;
+        v[q] = second[g];
+        ph[q] = phi[g];
+        vv[q] = V[g];
+        if constexpr (KEEP) pq[q] = v[q];
+      }
+    } else {  // the refinement's state: inside a solve only
 #pragma unroll
       for (int q = 0; q < E; ++q) {
         const long long g = base + t + q * Tl;
         ph[q] = phi[g];
         vv[q] = V[g];
-        if (a.solver) pq[q] = p[g];
-        else v[q] = cconv<TF>(a.f ? f[g] : ph[q]);
+        pq[q] = p[g];
       }
     }
     if (!RES && a.solver) {
@@ -810,7 +826,9 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
 #pragma unroll
       for (int q = 0; q < E; ++q) {
         if (retract) {
-          const CD d = pq[q];
+          CD d;
+          if constexpr (ONE) d = v[q];
+          else d = pq[q];
           ph[q] = cmk<CS>(cc * ph[q].x + mul_sd<TS>(ss, d.x), cc * ph[q].y + mul_sd<TS>(ss, d.y));
           phi_out[base + t + q * Tl] = ph[q];
         }
@@ -835,7 +853,11 @@ __device__ __forceinline__ void xunit(const PassArgs& a, const Scal& S, long lon
         const long long g = base + t + q * Tl;
         const TS u = ph[q].x * ph[q].x + ph[q].y * ph[q].y;
         const TS m = vv[q] + eta * u;
-        const CS fq = (a.f && !a.solver) ? f[g] : ph[q];  // the operand f (re-read in API mode)
+        CS fq = ph[q];
+        if (!a.solver) {
+          if constexpr (KEEP) fq = pq[q];
+          else if (a.f) fq = f[g];
+        }
         tout[g] = cmk<CS>(TS(v[q].x) + m * fq.x, TS(v[q].y) + m * fq.y);
       }
     }
