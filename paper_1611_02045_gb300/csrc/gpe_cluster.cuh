@@ -57,11 +57,18 @@ template <typename T, int M> struct ClusterHSmem {
   static constexpr size_t bytes = (size_t)(2 * kClusterRows * M + kClusterRows * LS) * sizeof(cplx<T>);
 };
 
+// Complex128 at M = 128: two CTAs fit an SM's shared memory (100 KB each) and, held to 128
+// registers, its register file too; with the 136 it takes alone, 49 fields took 220 us
+// instead of 185.  M = 256 fills the shared memory with one, smaller M stay below 128.
+template <typename T, int M> struct ClusterHMinBlocks {
+  static constexpr int value = sizeof(T) == 8 && M == 128 ? 2 : ClusterMinBlocks<T>::value;
+};
+
 // EV values per thread: 8 (radix-8 then 8/4/2 Stockham stages, two exchanges
 // per 256-point transform) or 16 (radix-16 stages: one exchange, half the
 // shared-memory traffic, half the threads).
 template <typename T, int M, int EV>
-__global__ void __launch_bounds__((M / EV) * kClusterRows, ClusterMinBlocks<T>::value) cluster_apply_H(const __grid_constant__ ClusterHArgs a) {
+__global__ void __launch_bounds__((M / EV) * kClusterRows, ClusterHMinBlocks<T, M>::value) cluster_apply_H(const __grid_constant__ ClusterHArgs a) {
   using C = cplx<T>;
   constexpr int E = EV, Tl = M / EV, R = kClusterRows;
   constexpr int LS = ClusterHSmem<T, M>::LS;
