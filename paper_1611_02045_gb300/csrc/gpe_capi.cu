@@ -139,7 +139,8 @@ static bool is_device_ptr(const void* p) {
 //  * width: the widest block up to the thread cap, halved while the axis has fewer
 //    than 128 blocks and the block more than one warp: blocks below a warp waste
 //    lanes, and every block costs a ticket and a partial (32^3 with blocks of 8
-//    threads: 158 us per complex64 iteration against 79 with these widths).  Strided
+//    threads: 158 us per complex64 iteration; with these widths, and the partials summed
+//    in parallel, 64).  Strided
 //    tiles have up to 16 columns, those of lines below 64 points up to 128 threads: with
 //    16 columns the z pass of 256 x 128 x 16 has 2048 blocks of a warp, whose partials
 //    the last one sums alone (gpe_energy, complex64: 93 us against 57 with 64 columns).

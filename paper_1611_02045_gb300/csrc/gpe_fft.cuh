@@ -193,7 +193,7 @@ template <int R, int DIR, typename C> __device__ __forceinline__ void dft_small(
 // eighth of their operations) and in a last radix 2 or 4 behind two radix-8 stages; in
 // M = 16 and 32 it would gain little.  The cascade takes as few operations with four
 // table entries instead of seven, and is 2% faster (H phi on 128^3 complex128 519 against
-// 531 us), but multiplies every value three times.  Measured, H f along one axis, error
+// 529 us), but multiplies every value three times.  Measured, H f along one axis, error
 // in 2^-53 (twiddles from rounded angles and cascaded -> as it is): M = 128 2.56 -> 2.31
 // and (E = 4) 2.88 -> 2.25, M = 512 3.03 -> 2.79 and 3.39 -> 2.57; products apart and
 // rounded angles: 2.67, 2.52, 3.10, 3.04.

@@ -1125,9 +1125,9 @@ __device__ __forceinline__ void sunit(const PassArgs& a, const Scal& S, long lon
 // sums every region of the operator in a fixed order and runs the scalar step
 // on a copy of the control block in shared memory: read once, written back
 // once, instead of a memory round trip per scalar.  Passes look at `done` only
-// once their operands are in flight.  Together with the shorter scalar steps and
-// the scalars split once (Num), an iteration of the graph loop went from 82 to 71
-// us (256^2, complex64), 121 to 113 us (256^2, refinement) and 585 to 531 us
+// once their operands are in flight.  With the shorter scalar steps, the scalars
+// split once (Num), the short sums above and four values per thread, an iteration of
+// the graph loop went from 121 to 74 us (256^2, refinement) and from 585 to 445 us
 // (128^3, refinement).
 // ---------------------------------------------------------------------------
 // All the sums of ROLE's operator, in the order its scalar step reads them: those of
